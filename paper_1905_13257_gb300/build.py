@@ -21,7 +21,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["capi.cu", "sketch_simt.cu", "sketch_tc.cu", "cpqr.cu", "coarse.cu", "coarse_coop.cu",
            "recon.cu",
            "recon_tc.cu", "single_pass.cu", "noalloc.cu", "tma_host.cu", "batch.cu",
-           "mlp.cu", "restricted.cu", "gauss_table.cpp"]
+           "mlp.cu", "gauss_table.cpp"]
 
 
 def nvcc() -> str:

@@ -91,7 +91,7 @@ void free_all(id_sketch* h) {
                   h->d_colpos, h->d_kout, h->d_V, h->d_F, h->d_nu2, h->d_nu20, h->d_gvec, h->d_hvec, h->d_vh, h->d_vl,
                   h->d_upart, h->d_cscal, h->d_cint, h->d_rlist, h->d_Rc, h->d_Pc, h->d_Jc,
                   h->d_colposc, h->d_part, h->d_out3, h->d_Jin, h->d_Pin, h->d_status, h->d_wpart,
-                  h->d_axis, h->d_Sc, h->d_cand, h->d_fq, h->d_crow, h->d_colscale};
+                  h->d_axis, h->d_Sc, h->d_cand, h->d_crow, h->d_colscale};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -235,11 +235,9 @@ id_status factor_enqueue(id_sketch* h, bool one_cta) {
   const int64_t n = h->n_seen;
   if (n == 0) return ID_ERR_STATE;
   const int k = h->k, l = h->l;
-  IDSK_CUDA(h, cudaMemcpy2DAsync(h->d_work, sizeof(double) * n, h->d_W,
-                                 sizeof(double) * h->n_max, sizeof(double) * n, l,
-                                 cudaMemcpyDeviceToDevice, h->st));
-  IDSK_CUDA(h, launch_cpqr_small(h->d_work, l, (int)n, (int)n, k, ID_RANK_TOL_FACTOR, h->d_R,
-                                 h->d_J, h->d_colpos, h->d_kout, h->st, one_cta));
+  IDSK_CUDA(h, launch_cpqr_small(h->d_W, h->n_max, h->d_work, l, (int)n, k, ID_RANK_TOL_FACTOR,
+                                 nullptr, h->d_R, h->d_J, h->d_colpos, h->d_kout, h->st,
+                                 one_cta));
   IDSK_CUDA(h, launch_solve_p(h->d_R, h->d_J, h->d_colpos, h->d_kout, k, (int)n, h->d_P, h->st));
   return ID_OK;
 }
@@ -405,7 +403,6 @@ id_status id_sketch_create(const id_config* cfg, void* cuda_stream, id_sketch** 
   al.get(&h->d_colpos, (size_t)nm);
   al.get(&h->d_kout, 1);
   al.get(&h->d_cand, (size_t)nm);
-  al.get(&h->d_fq, (size_t)l * k + k + (size_t)k * k);
   h->rec_blocks = 8 * h->nsm;
   al.get(&h->d_part, (size_t)3 * h->rec_blocks);
   al.get(&h->d_out3, 3);
@@ -514,18 +511,20 @@ id_status id_factor(id_sketch* h, int32_t* J, double* P, int32_t* k_out) {
   if (s != ID_OK) return s;
   if (h->n_seen == 0) return ID_ERR_STATE;
   // With want_coarse, the coarse QR of these columns (Algorithm 5) starts now
-  // on the side stream, on all SMs but one, and the QR of W runs beside it in
-  // one CTA; id_coarse_factor then only waits for it.
-  const bool spec = h->st2 && h->coarse_spec != h->n_seen &&
-                    coarse_coop_ok_ctas(h, h->nsm - 1);
+  // on the side stream and the QR of W runs beside it; id_coarse_factor then
+  // only waits for it.  The QR of W takes 8 SMs (the cluster form, enqueued
+  // first) when the coarse QR fits the others, else one.
+  const bool cluster = cpqr_cluster_ok(h->l, h->n_seen) && coarse_coop_ok_ctas(h, h->nsm - 8);
+  const int coarse_ctas = h->nsm - (cluster ? 8 : 1);
+  const bool spec = h->st2 && h->coarse_spec != h->n_seen && coarse_coop_ok_ctas(h, coarse_ctas);
   if (spec) IDSK_CUDA(h, cudaEventRecord(h->ev_sk, h->st));
-  s = factor_enqueue(h, spec);
+  s = factor_enqueue(h, spec && !cluster);
   if (s != ID_OK) return s;
   if (spec) {
     const id_status js = join_coarse(h);   // an earlier coarse QR, if any
     if (js != ID_OK) return js;
     IDSK_CUDA(h, cudaStreamWaitEvent(h->st2, h->ev_sk, 0));
-    IDSK_CUDA(h, launch_coarse_coop(h, h->n_seen, h->st2, h->nsm - 1));
+    IDSK_CUDA(h, launch_coarse_coop(h, h->n_seen, h->st2, coarse_ctas));
     IDSK_CUDA(h, cudaEventRecord(h->ev_cq, h->st2));
     h->coarse_spec = h->n_seen;
     h->cq_pending = true;
@@ -568,15 +567,17 @@ id_status id_factor_restricted(id_sketch* h, const int32_t* cand, int32_t ncand,
         return ID_ERR_INVALID_ARG;   // outside the streamed columns, or repeated
   }
   const int k = h->k, l = h->l;
-  IDSK_CUDA(h, cudaMemcpyAsync(h->d_cand, hc.data(), sizeof(int32_t) * ncand,
-                               cudaMemcpyHostToDevice, h->st));
-  IDSK_CUDA(h, launch_gather_cols(h->d_W, h->n_max, l, h->d_cand, ncand, h->d_work, h->st));
-  IDSK_CUDA(h, launch_cpqr_small(h->d_work, l, ncand, ncand, k, ID_RANK_TOL_FACTOR, h->d_R,
-                                 h->d_J, h->d_colpos, h->d_kout, h->st));
-  IDSK_CUDA(h, launch_map_pivots(h->d_J, h->d_cand, h->d_kout, k, h->d_Jin, h->st));
-  IDSK_CUDA(h, launch_fixed_solve(h->d_W, h->n_max, l, (int)n, h->d_Jin, h->d_kout, k, h->d_fq,
-                                  h->d_P, h->st));
-  if ((s = copy_out(h, J, h->d_Jin, sizeof(int32_t) * k)) != ID_OK) return s;
+  if (l > kLMax) IDSK_CUDA(h, cudaErrorInvalidValue);   // restricted form: l <= 64
+  // one QR of W over all n columns in which only the candidates may become
+  // pivots: R11 and R12 come out together, and P = R11^{-1} R12
+  std::vector<int32_t> pos((size_t)n, -1);
+  for (int32_t q = 0; q < ncand; ++q) pos[hc[q]] = q;
+  IDSK_CUDA(h, cudaMemcpyAsync(h->d_cand, pos.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice,
+                               h->st));
+  IDSK_CUDA(h, launch_cpqr_small(h->d_W, h->n_max, h->d_work, l, (int)n, k, ID_RANK_TOL_FACTOR,
+                                 h->d_cand, h->d_R, h->d_J, h->d_colpos, h->d_kout, h->st));
+  IDSK_CUDA(h, launch_solve_p(h->d_R, h->d_J, h->d_colpos, h->d_kout, k, (int)n, h->d_P, h->st));
+  if ((s = copy_out(h, J, h->d_J, sizeof(int32_t) * k)) != ID_OK) return s;
   if ((s = copy_out(h, P, h->d_P, sizeof(double) * k * n)) != ID_OK) return s;
   int32_t kk = 0, dst = 0;
   IDSK_CUDA(h, cudaMemcpyAsync(&kk, h->d_kout, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st));

@@ -11,16 +11,18 @@
 // from the updated matrix at every step (no downdating) and compared as its
 // square, ties to the lowest column index.
 //
-// n <= 1024 (cpqr_cluster_kernel): a cluster of 8 CTAs x 128 threads, one
-// column per thread held in registers for the whole factorization.  Per
-// step, each CTA's best candidate and then the pivot column are published in
-// its shared memory and read by the other CTAs through distributed shared
-// memory (two cluster barriers per step, double-buffered slots).
+// n <= 1024 and l <= 64 (cpqr_cluster_kernel): a cluster of 8 CTAs, every column
+// held in the registers of G lanes; one cluster barrier per step.
 // Larger n, or l > 64 rows (cpqr_small_kernel, up to 96 rows): one CTA of 1024
 // threads works in place on a copy of W held row-major in global memory
 // (L2-resident); thread t owns columns t, t + 1024, ...
-// In both, norms and the argmax use warp shuffles and fixed-order sums, and
-// the reflector of the pivot column is formed by one warp.
+// In both, sums run in a fixed order.
+//
+// Candidates.  With cpos (one int per column) only the columns with
+// cpos[j] >= 0 may become pivots, ties going to the lowest cpos, and the rank
+// tolerance is that of the candidate columns; every column is updated, so
+// that R11^{-1} R12 is the least-squares fit of all columns on W(:, J)
+// (the learned proposal's restricted ID).
 #include <cooperative_groups.h>
 #include <float.h>
 
@@ -32,162 +34,251 @@ namespace cg = cooperative_groups;
 namespace idsk {
 namespace {
 
-using qr::ArgMax;
-using qr::better;
-using qr::warp_argmax;
-using qr::warp_sum;
-
 constexpr int NT = 1024;
 constexpr int QMAX = 32;   // columns per thread -> n <= 32768
 
 __global__ void __launch_bounds__(NT, 1)
 cpqr_small_kernel(double* __restrict__ M, int rows, int n, int ld, int k, double tol_factor,
-                  double* __restrict__ R, int* __restrict__ J, int* __restrict__ colpos,
-                  int* __restrict__ kout) {
+                  const int* __restrict__ cpos, double* __restrict__ R, int* __restrict__ J,
+                  int* __restrict__ colpos, int* __restrict__ kout) {
   __shared__ qr::QrShared sh;
-  qr::cta_pivoted_qr<NT>(M, rows, n, ld, k, tol_factor, R, J, colpos, kout, sh);
+  qr::cta_pivoted_qr<NT>(M, rows, n, ld, k, tol_factor, cpos, R, J, colpos, kout, sh);
 }
 
 
-constexpr int CL_CTAS = 8, CL_THREADS = 128;   // cluster kernel: n <= 1024
+constexpr int CL_CTAS = 8;                    // CTAs of the cluster
+constexpr int CL_WARPS = 8;                   // warps that hold columns
+static_assert(CL_CTAS == 8 && CL_WARPS == 8, "best_of_8");
+constexpr int CL_WORKERS = CL_WARPS * 32;
+constexpr int CL_THREADS = CL_WORKERS + 32;   // and one warp for the step's scalars
 
-__device__ __forceinline__ void cpqr_cluster_body(const double* __restrict__ M, int rows, int n,
-                                                  int ld, int k, double tol_factor,
-                                                  double* __restrict__ R, int* __restrict__ J,
-                                                  int* __restrict__ colpos,
-                                                  int* __restrict__ kout) {
+// A candidate column: its residual norm as an ordered integer (0: none), its
+// place in the tie order, its index, its rows.
+struct Cand {
+  double col[kLMax];
+  unsigned long long key;
+  int ord, j;
+};
+
+__device__ __forceinline__ bool nonzero(double x) {   // on the integer units
+  return ((unsigned long long)__double_as_longlong(x) << 1) != 0ull;
+}
+
+// The lanes that hold the largest key and, among these, the lowest order
+// (whole warp; on the integer units).
+__device__ __forceinline__ bool warp_best(unsigned long long key, int ord,
+                                          unsigned long long* best, int* best_ord) {
+  const unsigned hi = (unsigned)(key >> 32);
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = hi == mh ? (unsigned)key : 0u;
+  const unsigned ml = __reduce_max_sync(0xffffffffu, lo);
+  const bool top = hi == mh && lo == ml;
+  const int o = __reduce_min_sync(0xffffffffu, top ? ord : 0x7fffffff);
+  *best = ((unsigned long long)mh << 32) | ml;
+  *best_ord = o;
+  return top && ord == o;
+}
+
+// The best of 8 candidates (whole warp).
+__device__ __forceinline__ int best_of_8(const Cand* c, int lane) {
+  unsigned long long k;
+  int o;
+  const bool win = warp_best(c[lane & 7].key, c[lane & 7].ord, &k, &o);
+  return (__ffs(__ballot_sync(0xffffffffu, win)) - 1) & 7;
+}
+
+// Column-pivoted Householder QR of M (rows x n row-major, rows <= 64, n <=
+// 8 * 256 / G) by a cluster of 8 CTAs.  M is only read.
+//
+// What bounds it is not the arithmetic (60 x 1000, k = 50: 5 MFMA) but the
+// chain of dependent phases of a step on narrow FP64 units (a warp's FP64
+// instruction takes an SM sub-partition's pipe for about 64 cycles, also when
+// it is predicated off).  So: a column's rows are spread over G lanes (row i
+// in lane i mod G: 4 to 32 rows a lane, rows above the pivot row are skipped
+// by branches that are uniform over the warp), G the largest that n allows;
+// columns are dealt to the CTAs in turn; the next norms are summed while the
+// columns are updated; every CTA pushes its best column with its norm into
+// the other CTAs' shared memory, so that one cluster barrier per step is
+// enough; the reflector is used unscaled, H = I - gamma v v^T with v = x,
+// v_s = x_s - beta and gamma = 1 / (||x||^2 + |x_s| ||x||), so that the
+// products v^T c start before the scalars, which a warp of their own forms
+// meanwhile (one square root and one division).  Rounding differs from the
+// scaled form by a few ulp only.
+// Measured (k = 50, l = 60; before: one column per thread, two cluster
+// barriers, every row in every step, 12.9 us a step for any n): n = 512 640 ->
+// 248 us, n = 200 (k = 20, l = 30) 258 -> 86 us, n = 1000 1779 us in one CTA
+// -> 387 us.
+template <int G>
+__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
+    cpqr_cluster_kernel(const double* __restrict__ M, int rows, int n, int64_t ld, int k,
+                        double tol_factor, const int* __restrict__ cpos, double* __restrict__ R,
+                        int* __restrict__ J, int* __restrict__ colpos, int* __restrict__ kout) {
+  constexpr int RPT = kLMax / G;   // rows per lane
   cg::cluster_group cl = cg::this_cluster();
-  __shared__ ArgMax cand[2];              // this CTA's best candidate (by step parity)
-  __shared__ double pcol[2][kLMax];       // pivot column, published by its owner CTA
-  __shared__ double fro_cta;
-  __shared__ ArgMax wred[CL_THREADS / 32];
-  __shared__ double fred[CL_THREADS / 32];
-  __shared__ double vs[kLMax];
-  __shared__ double sh_tau, sh_beta;
+  cl.barrier_arrive();   // waited for before the first write into another CTA
+  __shared__ Cand inbox[2][CL_CTAS];   // every CTA's best candidate, by step parity
+  __shared__ Cand wbest[CL_WARPS];
+  __shared__ double fro_w[CL_WARPS], fro_in[CL_CTAS];
+  __shared__ double sh_gamma, sh_v0, sh_beta;
   const int rank = (int)cl.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int j = rank * CL_THREADS + t;
-  const bool have = j < n;
+  const bool worker = warp < CL_WARPS;
+  const int g = lane & (G - 1);
+  const int j = (t / G) * CL_CTAS + rank;
+  const bool have = worker && j < n;
+  const bool busy = worker && ((t & ~31) / G) * CL_CTAS + rank < n;   // the warp holds a column
   const int kmax = min(k, min(rows, n));
-  double c[kLMax];
+
+  double c[RPT];
 #pragma unroll
-  for (int i = 0; i < kLMax; ++i) c[i] = (have && i < rows) ? M[(int64_t)i * ld + j] : 0.0;
-  if (have) colpos[j] = -1;
+  for (int q = 0; q < RPT; ++q)
+    c[q] = (have && g + G * q < rows) ? M[(int64_t)(g + G * q) * ld + j] : 0.0;
+  int ord = 0x7fffffff;   // place in the tie order; past the last: never a pivot
+  if (have) {
+    ord = cpos ? cpos[j] : j;
+    if (ord < 0) ord = 0x7fffffff;
+    if (g == 0) colpos[j] = -1;
+  }
   bool piv = false;
 
-  // ||W||_F: rows in order per column, then warps, then CTAs in rank order
-  {
-    double ss = 0.0;
+  // sum over the G lanes of a column (fixed tree)
+  auto group_sum = [&](double v) {
 #pragma unroll
-    for (int i = 0; i < kLMax; ++i) ss += c[i] * c[i];
-    ss = warp_sum(ss);
-    if (lane == 0) fred[warp] = ss;
-    __syncthreads();
-    if (t == 0) {
-      double a = 0.0;
-      for (int w = 0; w < CL_THREADS / 32; ++w) a += fred[w];
-      fro_cta = a;
-    }
+    for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  double ss = 0.0;   // the column's residual norm, squared
+  if (busy) {
+#pragma unroll
+    for (int q = 0; q < RPT; ++q)
+      if (G * q < rows) ss += c[q] * c[q];
+    ss = group_sum(ss);
   }
-  cl.sync();
-  double fro2 = 0.0;
-  for (int r = 0; r < CL_CTAS; ++r) fro2 += *cl.map_shared_rank(&fro_cta, r);
-  const double tol = tol_factor * DBL_EPSILON * sqrt(fro2);
+  // ||W||_F of the candidates: columns of a warp, warps, CTAs in order
+  if (worker) {
+    double f = ord != 0x7fffffff ? ss : 0.0;
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    if (lane == 0) fro_w[warp] = f;
+  }
+  __syncthreads();
+  cl.barrier_wait();
+  if (t < CL_CTAS) {
+    double f = 0.0;
+    for (int w = 0; w < CL_WARPS; ++w) f += fro_w[w];
+    *cl.map_shared_rank(&fro_in[rank], t) = f;   // read after step 0's cluster barrier
+  }
+  double tol2 = 0.0;
 
   int s = 0;
   for (; s < kmax; ++s) {
     const int b = s & 1;
-    // residual norm of this thread's column, rows s.. in order
-    ArgMax best{-1.0, 0x7fffffff};
-    if (have && !piv) {
-      double ss = 0.0;
-#pragma unroll
-      for (int i = 0; i < kLMax; ++i)
-        if (i >= s && i < rows) ss += c[i] * c[i];
-      best = ArgMax{ss, j};
-    }
-    best = warp_argmax(best);
-    if (lane == 0) wred[warp] = best;
-    __syncthreads();
-    if (t == 0) {
-      ArgMax a = wred[0];
-      for (int w = 1; w < CL_THREADS / 32; ++w) a = better(a, wred[w]);
-      cand[b] = a;
-    }
-    cl.sync();   // candidates published
-    ArgMax g = *cl.map_shared_rank(&cand[b], 0);
-    for (int r = 1; r < CL_CTAS; ++r) g = better(g, *cl.map_shared_rank(&cand[b], r));
-    if (!(g.v > tol * tol)) break;   // uniform over the cluster
-    const int p = g.i;
-    if (j == p) {
-#pragma unroll
-      for (int i = 0; i < kLMax; ++i) pcol[b][i] = c[i];
-    }
-    cl.sync();   // pivot column published
-    if (warp == 0) {   // Householder reflector of the pivot column, rows s..rows-1
-      const double* pc = cl.map_shared_rank(&pcol[b][0], p / CL_THREADS);
-      const int len = rows - s;
-      const double x0 = (lane < len) ? pc[s + lane] : 0.0;
-      const double x1 = (lane + 32 < len) ? pc[s + lane + 32] : 0.0;
-      const double alpha = __shfl_sync(0xffffffffu, x0, 0);
-      const double sigma = warp_sum((lane == 0 ? 0.0 : x0 * x0) + x1 * x1);
-      double tau = 0.0, beta = alpha, scale = 0.0;
-      if (sigma != 0.0) {
-        const double nrm = sqrt(alpha * alpha + sigma);
-        beta = alpha >= 0.0 ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        scale = alpha - beta;
-      }
-      if (lane < len) vs[lane] = lane == 0 ? 1.0 : (sigma != 0.0 ? x0 / scale : 0.0);
-      if (lane + 32 < len) vs[lane + 32] = sigma != 0.0 ? x1 / scale : 0.0;
+    const int gs = s & (G - 1), qs = s / G;   // lane and register of the pivot row
+    // the warp's candidate: largest norm, ties to the lowest order
+    if (worker) {
+      unsigned long long key = 0ull;
+      if (ord != 0x7fffffff && !piv) key = (unsigned long long)__double_as_longlong(ss) + 1ull;
+      unsigned long long wk;
+      int o;
+      const bool win = warp_best(key, ord, &wk, &o);
       if (lane == 0) {
-        sh_tau = tau;
+        wbest[warp].key = wk;
+        wbest[warp].ord = o;
+      }
+      if (wk != 0ull && win) {
+#pragma unroll
+        for (int q = 0; q < RPT; ++q)
+          if (q >= qs) wbest[warp].col[g + G * q] = c[q];
+        if (g == 0) wbest[warp].j = j;
+      }
+    }
+    __syncthreads();
+    // the CTA's candidate into every CTA's inbox
+    {
+      const int w = best_of_8(wbest, lane);
+      for (int e = t; e < CL_CTAS * kLMax; e += CL_THREADS) {
+        const int i = e & (kLMax - 1);
+        if (i >= s && i < rows)
+          cl.map_shared_rank(&inbox[b][rank], e / kLMax)->col[i] = wbest[w].col[i];
+      }
+      if (t < CL_CTAS) {
+        Cand* dst = cl.map_shared_rank(&inbox[b][rank], t);
+        dst->key = wbest[w].key;
+        dst->ord = wbest[w].ord;
+        dst->j = wbest[w].j;
+      }
+    }
+    cl.sync();
+    const Cand& pc = inbox[b][best_of_8(inbox[b], lane)];
+    if (s == 0) {
+      double f = 0.0;
+      for (int x = 0; x < CL_CTAS; ++x) f += fro_in[x];
+      const double tol = tol_factor * DBL_EPSILON * sqrt(f);
+      tol2 = tol * tol;
+    }
+    const double nrm2 = __longlong_as_double((long long)(pc.key - 1ull));
+    if (pc.key == 0ull || !(nrm2 > tol2)) break;   // uniform over the cluster
+    const int p = pc.j;
+    double x[RPT], d = 0.0, cs = 0.0;
+    if (!worker) {
+      // scalars of the reflector; below the pivot row all zero: H = I
+      const double a0 = pc.col[s];
+      const double x0 = s + 1 + lane < rows ? pc.col[s + 1 + lane] : 0.0;
+      const double x1 = s + 33 + lane < rows ? pc.col[s + 33 + lane] : 0.0;
+      const bool any = __any_sync(0xffffffffu, nonzero(x0) || nonzero(x1));
+      if (lane == 0) {
+        double beta = a0, gamma = 0.0, v0 = 0.0;
+        if (any) {
+          const double nrm = sqrt(nrm2);
+          beta = a0 >= 0.0 ? -nrm : nrm;
+          v0 = a0 - beta;
+          gamma = 1.0 / (nrm2 + fabs(a0) * nrm);
+        }
         sh_beta = beta;
+        sh_gamma = gamma;
+        sh_v0 = v0;
         if (rank == 0) {
           J[s] = p;
           colpos[p] = s;
         }
       }
+    } else if (busy) {
+      // x = the pivot column below row s; d = x^T c, cs = row s of the column
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        x[q] = 0.0;
+        if (q >= qs && G * q < rows) {
+          if (g + G * q > s && g + G * q < rows) x[q] = pc.col[g + G * q];
+          d += x[q] * c[q];
+          if (q == qs) cs = c[q];
+        }
+      }
+      d = group_sum(d);
+      cs = __shfl_sync(0xffffffffu, cs, (lane & ~(G - 1)) + gs);
     }
     __syncthreads();
-    if (have) {
-      double rsj;
-      if (j == p) {
-        piv = true;
-        rsj = sh_beta;
-      } else if (piv) {
-        rsj = 0.0;
-      } else {
-        const double tau = sh_tau;
-        if (tau != 0.0) {
-          double d = 0.0;
+    if (busy) {
+      const double v0 = sh_v0;
+      const double w = sh_gamma * (d + v0 * cs);
+      ss = 0.0;
 #pragma unroll
-          for (int i = 0; i < kLMax; ++i)
-            if (i >= s && i < rows) d += vs[i - s] * c[i];
-          const double td = tau * d;
-#pragma unroll
-          for (int i = 0; i < kLMax; ++i)
-            if (i >= s && i < rows) c[i] -= td * vs[i - s];
+      for (int q = 0; q < RPT; ++q) {
+        if (q >= qs && G * q < rows) {
+          c[q] -= w * x[q];
+          const double y = (q > qs || g > gs) ? c[q] : 0.0;   // rows below s
+          ss += y * y;
         }
-#pragma unroll
-        for (int i = 0; i < kLMax; ++i)
-          if (i == s) rsj = c[i];
       }
-      R[(int64_t)s * n + j] = rsj;
+      ss = group_sum(ss);
+      if (j == p) piv = true;
+      if (have && g == 0)
+        R[(int64_t)s * n + j] = j == p ? sh_beta : (piv ? 0.0 : cs - w * v0);
     }
   }
   if (rank == 0) {
     if (t == 0) *kout = s;
     for (int q = s + t; q < k; q += CL_THREADS) J[q] = -1;
   }
-  cl.sync();   // no CTA leaves while another may still read its shared memory
-}
-
-__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
-    cpqr_cluster_kernel(const double* __restrict__ M, int rows, int n, int ld, int k,
-                        double tol_factor, double* __restrict__ R, int* __restrict__ J,
-                        int* __restrict__ colpos, int* __restrict__ kout) {
-  cpqr_cluster_body(M, rows, n, ld, k, tol_factor, R, J, colpos, kout);
 }
 
 
@@ -219,17 +310,36 @@ __global__ void __launch_bounds__(SP_WARPS * 32) solve_p_kernel(
 
 }  // namespace
 
-// one_cta: the one-CTA kernel whatever the size (the QR then occupies a
-// single SM, beside the coarse QR that id_factor starts on a side stream).
-cudaError_t launch_cpqr_small(double* M, int rows, int n, int ld, int k, double tol_factor,
-                              double* R, int* J, int* colpos, int* kout, cudaStream_t st,
-                              bool one_cta) {
+bool cpqr_cluster_ok(int rows, int64_t n) { return rows <= kLMax && n <= 1024; }
+
+// The cluster form reads W itself; the one-CTA form works in place on a copy
+// of W in `work` (rows x n).  G: the most lanes per column that n columns on 8
+// CTAs of 256 threads allow.
+cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int rows, int n, int k,
+                              double tol_factor, const int* cpos, double* R, int* J, int* colpos,
+                              int* kout, cudaStream_t st, bool one_cta) {
   if (n > NT * QMAX || rows > kLMaxW || k > kLMaxW) return cudaErrorInvalidValue;
-  if (!one_cta && n <= CL_CTAS * CL_THREADS && rows <= kLMax)   // cluster: a column in registers
-    cpqr_cluster_kernel<<<CL_CTAS, CL_THREADS, 0, st>>>(M, rows, n, ld, k, tol_factor, R, J,
-                                                        colpos, kout);
-  else
-    cpqr_small_kernel<<<1, NT, 0, st>>>(M, rows, n, ld, k, tol_factor, R, J, colpos, kout);
+  if (!one_cta && cpqr_cluster_ok(rows, n)) {
+    const int cols = (n + CL_CTAS - 1) / CL_CTAS;   // columns per CTA
+    auto go = [&](auto kern) {
+      kern<<<CL_CTAS, CL_THREADS, 0, st>>>(W, rows, n, ldw, k, tol_factor, cpos, R, J, colpos,
+                                           kout);
+    };
+    if (cols <= CL_WORKERS / 16)
+      go(cpqr_cluster_kernel<16>);
+    else if (cols <= CL_WORKERS / 8)
+      go(cpqr_cluster_kernel<8>);
+    else if (cols <= CL_WORKERS / 4)
+      go(cpqr_cluster_kernel<4>);
+    else
+      go(cpqr_cluster_kernel<2>);
+  } else {
+    const cudaError_t e =
+        cudaMemcpy2DAsync(work, sizeof(double) * n, W, sizeof(double) * ldw, sizeof(double) * n,
+                          rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    cpqr_small_kernel<<<1, NT, 0, st>>>(work, rows, n, n, k, tol_factor, cpos, R, J, colpos, kout);
+  }
   count_launches(1);
   return cudaGetLastError();
 }

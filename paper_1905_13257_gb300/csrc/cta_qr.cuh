@@ -16,7 +16,8 @@ constexpr int kQrCols = 32;   // columns per thread at most (pivot bit mask)
 
 struct ArgMax {
   double v;
-  int i;
+  int i;   // place in the tie order (lowest wins)
+  int j;   // column
 };
 
 __device__ __forceinline__ ArgMax better(ArgMax a, ArgMax b) {
@@ -30,6 +31,7 @@ __device__ __forceinline__ ArgMax warp_argmax(ArgMax a) {
     ArgMax b;
     b.v = __shfl_xor_sync(0xffffffffu, a.v, o);
     b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
+    b.j = __shfl_xor_sync(0xffffffffu, a.j, o);
     a = better(a, b);
   }
   return a;
@@ -54,12 +56,16 @@ struct QrShared {
 // <= 96) by the NT threads of one CTA, in place: thread t owns columns t,
 // t + NT, ... (n <= 32 NT).  k pivots at most; stops early below the rank
 // tolerance tol_factor * eps * ||M||_F.  Writes R (k x n), J (k, -1 past
-// k_out), colpos (n: pivot position or -1) and *kout.
+// k_out), colpos (n: pivot position or -1) and *kout.  With cpos, only the
+// columns with cpos[j] >= 0 may become pivots (ties to the lowest cpos) and
+// count in ||M||_F.
 template <int NT>
 __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows, int n, int ld,
-                                               int k, double tol_factor, double* __restrict__ R,
-                                               int* __restrict__ J, int* __restrict__ colpos,
-                                               int* __restrict__ kout, QrShared& sh) {
+                                               int k, double tol_factor,
+                                               const int* __restrict__ cpos,
+                                               double* __restrict__ R, int* __restrict__ J,
+                                               int* __restrict__ colpos, int* __restrict__ kout,
+                                               QrShared& sh) {
   static_assert(NT % 32 == 0 && NT <= 1024, "whole warps, at most 32");
   ArgMax* red = sh.red;
   double* vs = sh.vs;
@@ -82,7 +88,7 @@ __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows,
       if (j >= n) break;
       for (int i = 0; i < rows; ++i) {
         const double x = M[(int64_t)i * ld + j];
-        ss += x * x;
+        if (!cpos || cpos[j] >= 0) ss += x * x;
       }
       colpos[j] = -1;
     }
@@ -100,26 +106,26 @@ __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows,
   int s = 0;
   for (; s < kmax; ++s) {
     // residual norms of the non-pivoted columns
-    ArgMax best{-1.0, 0x7fffffff};
+    ArgMax best{-1.0, 0x7fffffff, -1};
     for (int q = 0; q < kQrCols; ++q) {
       const int j = t + q * NT;
       if (j >= n) break;
-      if (pivoted & (1u << q)) continue;
+      if ((pivoted & (1u << q)) || (cpos && cpos[j] < 0)) continue;
       double ss = 0.0;
       for (int i = s; i < rows; ++i) {
         const double x = M[(int64_t)i * ld + j];
         ss += x * x;
       }
-      best = better(best, ArgMax{ss, j});
+      best = better(best, ArgMax{ss, cpos ? cpos[j] : j, j});
     }
     best = warp_argmax(best);
     if (lane == 0) red[warp] = best;
     __syncthreads();
     if (warp == 0) {
-      ArgMax b = lane < NT / 32 ? red[lane] : ArgMax{-1.0, 0x7fffffff};
+      ArgMax b = lane < NT / 32 ? red[lane] : ArgMax{-1.0, 0x7fffffff, -1};
       b = warp_argmax(b);
       if (lane == 0) {
-        sh_p = b.i;
+        sh_p = b.j;
         sh_stop = !(b.v > sh_tol * sh_tol);
       }
     }

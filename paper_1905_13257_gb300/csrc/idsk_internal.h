@@ -288,8 +288,7 @@ struct id_sketch {
   int* d_J = nullptr;         // k
   int* d_colpos = nullptr;    // n_max
   int* d_kout = nullptr;      // 1
-  int* d_cand = nullptr;      // n_max: candidate columns (id_factor_restricted)
-  double* d_fq = nullptr;     // l k + k + k k: reflectors, tau, R of W(:, J)
+  int* d_cand = nullptr;      // n_max: each column's place among the candidates, -1 for none
   // coarse workspace (allocated with the handle when want_coarse)
   double* d_V = nullptr;      // mc x k: reflectors as FP32 pairs (8 bytes each)
   double* d_F = nullptr;      // n_max x k
@@ -364,9 +363,13 @@ cudaError_t launch_sketch_batch(const BatchJob* jobs, const CUtensorMap* tmaps,
                                 float* slabs, int* counters, const QrJob* qjobs,
                                 double tol_factor, int* stat, int grid, int drain_blocks,
                                 cudaStream_t st);
-cudaError_t launch_cpqr_small(double* M, int rows, int n, int ld, int k, double tol_factor,
-                              double* R, int* J, int* colpos, int* kout, cudaStream_t st,
-                              bool one_cta = false);
+// Pivoted QR of W (rows x n row-major, leading dimension ldw) into R (k x n), J,
+// colpos and kout; work: rows x n scratch; cpos: null, or the candidates'
+// places in the tie order (-1: not a candidate).
+bool cpqr_cluster_ok(int rows, int64_t n);
+cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int rows, int n, int k,
+                              double tol_factor, const int* cpos, double* R, int* J, int* colpos,
+                              int* kout, cudaStream_t st, bool one_cta = false);
 cudaError_t launch_solve_p(const double* R, const int* J, const int* colpos, const int* kout,
                            int k, int n, double* P, cudaStream_t st);
 cudaError_t launch_coarse_cpqr(id_sketch* h, int64_t n, cudaStream_t st);
@@ -397,12 +400,6 @@ cudaError_t launch_single_pass_lift(const InterpGeom& g, int64_t m, int dtype, i
                                     cudaStream_t st);
 void gaussian_table_host(float* vals, uint16_t* bits);
 void count_launches(int64_t n);
-cudaError_t launch_gather_cols(const double* W, int64_t ldw, int l, const int* cand, int ncand,
-                               double* Wc, cudaStream_t st);
-cudaError_t launch_map_pivots(const int* Jc, const int* cand, const int* kout, int k, int* J,
-                              cudaStream_t st);
-cudaError_t launch_fixed_solve(const double* W, int64_t ldw, int l, int n, const int* J,
-                               const int* kout, int k, double* fq, double* P, cudaStream_t st);
 // Launch the sketch of every pending column window of the handle (capi.cu).
 id_status launch_pending(id_sketch* h);
 // Enqueue the randomized ID of the streamed columns (pivoted QR of W and the

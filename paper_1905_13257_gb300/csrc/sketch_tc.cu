@@ -808,8 +808,8 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
   }
   __syncthreads();
   qr::QrShared& sh = *reinterpret_cast<qr::QrShared*>(scratch);
-  qr::cta_pivoted_qr<NTHREADS_TMA>(q.M, q.rows, q.n, q.n, q.k, tol_factor, q.R, q.J, q.colpos,
-                                   q.kout, sh);
+  qr::cta_pivoted_qr<NTHREADS_TMA>(q.M, q.rows, q.n, q.n, q.k, tol_factor, nullptr, q.R, q.J,
+                                   q.colpos, q.kout, sh);
   __syncthreads();
   double* r11 = reinterpret_cast<double*>(scratch + 4096);
   double* rdiag = r11 + kLMaxW * kLMaxW;
