@@ -171,7 +171,7 @@ id_status launch_pending(id_sketch* h) {
     if (!tc && h->l > kLMax) return ID_ERR_UNSUPPORTED;   // wide sketches: tensor-core path only
     const bool fp8 = h->cfg.prec == ID_SKETCH_FP8E4M3;
     if (!tc && fp8) return ID_ERR_UNSUPPORTED;             // FP8 form: tensor-core path only
-    const int wmax = tc ? kTcMaxTiles * 128 : kSimtWindowMax;
+    const int wmax = tc ? kTcMaxTiles * 128 : simt_window_cols(h->l, h->cfg.dtype);
     int taken = 0;
     size_t consumed = 0;
     while (consumed < h->pend.size() && w.nseg < kMaxSegs && taken < wmax) {

@@ -20,7 +20,7 @@ constexpr int kLMax = 64;             // sketch width l (padded to 16 on device)
 constexpr int kLMaxW = 96;
 constexpr int kPassRows = 60;         // a multiple of 10: Psi's counter blocks
 constexpr int kMaxSegs = 64;          // column segments per sketch launch
-constexpr int kSimtWindowMax = 320;   // columns per SIMT sketch launch
+constexpr int kSimtWindowMax = 320;   // columns per SIMT sketch launch at most
 constexpr int kTcMaxTiles = 4;        // 128-column tiles per tensor-core launch (TMEM budget)
 constexpr int kRecKMax = 64;          // rank handled by the error pass
 constexpr int kTableSize = 4096;
@@ -347,6 +347,7 @@ cudaError_t launch_fp8_scales(const Window& w, int64_t m, float* scale, cudaStre
 cudaError_t launch_gaussian_fill(uint32_t which, uint32_t k0, uint32_t k1, int64_t first,
                                  int64_t count, int width, const float* table, float* out,
                                  cudaStream_t st);
+int simt_window_cols(int l, int dtype);   // columns of one SIMT sketch launch at most
 cudaError_t launch_sketch_simt(const SketchArgs& a, const Window& w, int dtype, int nsm,
                                cudaStream_t st);
 cudaError_t launch_sketch_tc(const SketchArgs& a, const Window& w, int npieces, int nsm,
