@@ -151,10 +151,11 @@ id_status id_sketch_reset(id_sketch* h);
  * to the lowest column index.
  * Returns ID_ERR_RANK_DEFICIENT when fewer than k pivots clear the rank
  * tolerance; J and the first k_out rows of P are still valid.
- * With want_coarse (FP32 data, cooperative coarse QR), the call also starts
- * id_coarse_factor's QR of the same columns on an internal stream of the
- * handle, on all SMs but one, and runs the QR of W in one CTA beside it; it
- * returns when J, P and k_out are ready.  The handle orders that work before
+ * With want_coarse (cooperative coarse QR: at most 512 coarse rows per SM), the
+ * call also starts id_coarse_factor's QR of the same columns on an internal
+ * stream of the handle, on the SMs that the QR of W leaves (all but 8, or but
+ * one when those cannot hold the coarse rows); it returns when J, P and k_out
+ * are ready.  The handle orders that work before
  * anything that would overwrite its inputs (new columns, a reset).
  * Errors: ID_ERR_STATE when no column was streamed. */
 id_status id_factor(id_sketch* h, int32_t* J, double* P, int32_t* k_out);

@@ -414,7 +414,7 @@ id_status id_sketch_create(const id_config* cfg, void* cuda_stream, id_sketch** 
     al.get(&h->d_nu2, (size_t)nm);
     al.get(&h->d_nu20, (size_t)nm);
     al.get(&h->d_gvec, (size_t)h->coarse_blocks * nm);            // row-range partials of A_c^T u
-    al.get(&h->d_hvec, (size_t)kLMax);                             // V_s^T v_s
+    al.get(&h->d_hvec, (size_t)kLMax + 1);                         // V_s^T v_s; row s of V, u_s
     al.get(&h->d_vh, (size_t)h->mc + 8);                           // u below row s, FP32 pair
     al.get(&h->d_vl, (size_t)h->mc + 8);
     al.get(&h->d_upart, (size_t)h->coarse_blocks * (kLMax + 1));   // V_s^T u, ||u||^2 partials
@@ -437,8 +437,7 @@ id_status id_sketch_create(const id_config* cfg, void* cuda_stream, id_sketch** 
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_status, 0, sizeof(int), h->st);
   if (e == cudaSuccess && h->d_crow) e = launch_coarse_rows(h->cg, h->m, h->d_crow, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-  if (e == cudaSuccess && cfg->want_coarse && cfg->dtype == ID_F32 &&
-      !getenv("IDSKETCH_NO_SIDE_STREAM")) {
+  if (e == cudaSuccess && cfg->want_coarse && !getenv("IDSKETCH_NO_SIDE_STREAM")) {
     e = cudaStreamCreateWithFlags(&h->st2, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_sk, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_cq, cudaEventDisableTiming);

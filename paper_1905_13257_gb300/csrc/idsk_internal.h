@@ -295,7 +295,7 @@ struct id_sketch {
   double* d_nu2 = nullptr;    // n_max
   double* d_nu20 = nullptr;   // n_max
   double* d_gvec = nullptr;   // coarse_blocks x n_max: row-range partials of A_c^T u
-  double* d_hvec = nullptr;   // kLMax: V_s^T v_s
+  double* d_hvec = nullptr;   // kLMax + 1: V_s^T v_s; row s of V and u_s (cooperative form)
   float* d_vh = nullptr;      // mc: u below row s as an FP32 pair (hi)
   float* d_vl = nullptr;      // mc: (lo)
   double* d_upart = nullptr;  // coarse_blocks x (kLMax + 1): partials of V_s^T u, ||u||^2
@@ -308,8 +308,8 @@ struct id_sketch {
   int* d_colposc = nullptr;   // n_max
   int coarse_blocks = 0;
   // The coarse QR of the same columns started by id_factor on a side stream
-  // (want_coarse, FP32, cooperative form): it runs beside the small QR of W
-  // and id_coarse_factor only waits for it.
+  // (want_coarse, cooperative form): it runs beside the small QR of W and
+  // id_coarse_factor only waits for it.
   cudaStream_t st2 = nullptr;     // side stream (created with the handle)
   cudaEvent_t ev_sk = nullptr;    // the sketch of the columns is complete
   cudaEvent_t ev_cq = nullptr;    // the side stream's coarse QR is complete
@@ -374,8 +374,8 @@ cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int ro
 cudaError_t launch_solve_p(const double* R, const int* J, const int* colpos, const int* kout,
                            int k, int n, double* P, cudaStream_t st);
 cudaError_t launch_coarse_cpqr(id_sketch* h, int64_t n, cudaStream_t st);
-// The coarse QR as one cooperative launch (coarse_coop.cu): FP32 A_c, m_c a
-// multiple of 4, at most 512 rows per CTA.
+// The coarse QR as one cooperative launch (coarse_coop.cu): at most 512 rows
+// of A_c per CTA.
 bool coarse_coop_ok(const id_sketch* h);
 cudaError_t launch_coarse_coop(id_sketch* h, int64_t n, cudaStream_t st, int max_ctas = 0);
 bool coarse_coop_ok_ctas(const id_sketch* h, int max_ctas);
