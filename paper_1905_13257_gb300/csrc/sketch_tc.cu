@@ -53,6 +53,7 @@
 // Every mbarrier wait is bounded: on timeout the CTA raises an abort flag,
 // every role leaves its loop, in-flight MMAs are waited for (bounded) and the
 // TMEM is freed; the host reads the status word and reports ID_ERR_TIMEOUT.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -66,6 +67,8 @@
 #include "df.cuh"
 #include "idsk_internal.h"
 #include "tc_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace idsk {
 namespace {
@@ -946,20 +949,46 @@ __global__ void wpart_reduce_kernel(const float* __restrict__ wpart, int nslab, 
 
 // FP8 form: per column of the window, the power of two 2^e with
 // max_r |A(r, c)| 2^e <= 448 < max_r |A(r, c)| 2^(e + 1) (e in [-100, 100];
-// 1 for a zero column), into scale[c].  One CTA per column.
-__global__ void fp8_scale_kernel(const __grid_constant__ Window w, int64_t m,
-                                 float* __restrict__ scale) {
-  __shared__ float red[32];
-  const int c = blockIdx.x;
-  const float* col = column_ptr(w, c);
+// 1 for a zero column), into scale[c].  One cluster of 8 CTAs per column, each
+// an eighth of its rows with 128-bit loads, eight in flight per thread; the
+// maxima meet in CTA 0 through distributed shared memory.  Bound by the one
+// read of the window: 1,797,120 x 500 (3.6 GB) 916 us with one CTA and one
+// scalar load at a time per column, 484 us now (7.4 TB/s).
+constexpr int FS_CTAS = 8, FS_THREADS = 256, FS_LOADS = 8;
+__global__ void __cluster_dims__(FS_CTAS, 1, 1) __launch_bounds__(FS_THREADS)
+    fp8_scale_kernel(const __grid_constant__ Window w, int64_t m, float* __restrict__ scale) {
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ float red[FS_THREADS / 32], cta_max;
+  const int c = blockIdx.y;
+  const float* col = column_ptr(w, c);   // 16-byte aligned
+  const int64_t q4 = m >> 2;             // whole row quads
+  const float4* col4 = reinterpret_cast<const float4*>(col);
+  const int64_t i1 = q4 * (blockIdx.x + 1) / FS_CTAS;
   float mx = 0.f;
-  for (int64_t r = threadIdx.x; r < m; r += blockDim.x) mx = fmaxf(mx, fabsf(col[r]));
+  auto take = [&](const float4& x) {
+    mx = fmaxf(fmaxf(fmaxf(mx, fabsf(x.x)), fmaxf(fabsf(x.y), fabsf(x.z))), fabsf(x.w));
+  };
+  int64_t i = q4 * blockIdx.x / FS_CTAS + threadIdx.x;
+  for (; i + (FS_LOADS - 1) * FS_THREADS < i1; i += FS_LOADS * FS_THREADS) {
+    float4 x[FS_LOADS];
+#pragma unroll
+    for (int u = 0; u < FS_LOADS; ++u) x[u] = __ldcs(col4 + i + u * FS_THREADS);
+#pragma unroll
+    for (int u = 0; u < FS_LOADS; ++u) take(x[u]);
+  }
+  for (; i < i1; i += FS_THREADS) take(__ldcs(col4 + i));
+  if (blockIdx.x == 0 && threadIdx.x < (m & 3)) mx = fmaxf(mx, fabsf(col[4 * q4 + threadIdx.x]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) mx = fmaxf(mx, red[i]);
+    for (int u = 1; u < FS_THREADS / 32; ++u) mx = fmaxf(mx, red[u]);
+    cta_max = mx;
+  }
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    for (int r = 1; r < FS_CTAS; ++r) mx = fmaxf(mx, *cl.map_shared_rank(&cta_max, r));
     int e = 0;
     if (mx > 0.f) {
       int p = 0;
@@ -971,6 +1000,7 @@ __global__ void fp8_scale_kernel(const __grid_constant__ Window w, int64_t m,
     }
     scale[c] = ldexpf(1.f, e);
   }
+  cl.sync();   // no CTA leaves before its maximum is read
 }
 
 template <int NP, bool TMA>
@@ -1118,7 +1148,7 @@ cudaError_t launch_coarse_rows(const CoarseGeom& g, int64_t m, int64_t* crow, cu
 
 cudaError_t launch_fp8_scales(const Window& w, int64_t m, float* scale, cudaStream_t st) {
   if (w.ncols <= 0) return cudaSuccess;
-  fp8_scale_kernel<<<w.ncols, 256, 0, st>>>(w, m, scale);
+  fp8_scale_kernel<<<dim3(FS_CTAS, (unsigned)w.ncols), FS_THREADS, 0, st>>>(w, m, scale);
   count_launches(1);
   return cudaGetLastError();
 }
