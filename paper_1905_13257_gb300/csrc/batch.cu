@@ -65,7 +65,7 @@ struct id_batch {
   int items_cap = 0;
   float* d_slabs = nullptr;
   size_t slab_cap = 0;                // floats
-  int* d_counter = nullptr;           // [0] the item counter, [1 + j] job j's completed items
+  int* d_counter = nullptr;           // the item counter
   QrJob* d_qr = nullptr;
   int item_mb = 0;                    // autotuned work-item size (0: automatic)
   int nsm = 0;
@@ -164,7 +164,6 @@ void build_jobs(id_batch* b) {
       j.ncols = p.n;
       j.np = j.a.bf16 ? 1 : 2;
       j.prob = (int)i;
-      j.Wd = h->d_work + (int64_t)s0 * p.n;
       b->jobs.push_back(j);
       b->tmaps.push_back(tm);
     }
@@ -202,22 +201,16 @@ id_status build_items(id_batch* b, int item_mb) {
     }
     j.nitem = (int32_t)items.size() - j.item0;
   }
-  // jobs in order of decreasing QR work (k n l), so that the QRs which the
-  // CTAs run as matrices complete overlap later items and the last matrices
-  // to complete have the cheapest ones; each job's items in row order
-  std::vector<int> jorder(b->jobs.size());
-  std::iota(jorder.begin(), jorder.end(), 0);
-  auto qr_work = [&](int q) {
-    const BatchJob& j = b->jobs[q];
-    return (double)b->prob[j.prob].k * j.ncols * j.a.l;
-  };
-  std::stable_sort(jorder.begin(), jorder.end(),
-                   [&](int x, int y) { return qr_work(x) > qr_work(y); });
-  std::vector<int32_t> order;
-  order.reserve(items.size());
-  for (int q : jorder)
-    for (int32_t it = b->jobs[q].item0; it < b->jobs[q].item0 + b->jobs[q].nitem; ++it)
-      order.push_back(it);
+  std::vector<int32_t> order(items.size());
+  std::iota(order.begin(), order.end(), 0);
+  // largest items first (a job's row blocks per item follow from its width, so
+  // the items differ by the ragged last ones only)
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    auto bytes = [&](int32_t i) {
+      return (double)items[i].nrb * b->jobs[items[i].job].ncols;
+    };
+    return bytes(x) > bytes(y);
+  });
   cudaError_t e = cudaSuccess;
   if ((int)items.size() > b->items_cap) {
     if (b->d_items) cudaFree(b->d_items);
@@ -239,7 +232,7 @@ id_status build_items(id_batch* b, int item_mb) {
   if (e == cudaSuccess && !b->d_jobs) {
     e = cudaMalloc(&b->d_jobs, sizeof(BatchJob) * b->jobs.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tmaps, sizeof(CUtensorMap) * b->tmaps.size());
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int) * (1 + b->jobs.size()));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_qr, sizeof(QrJob) * b->jobs.size());
     if (e == cudaSuccess)
       e = cudaMemcpy(b->d_tmaps, b->tmaps.data(), sizeof(CUtensorMap) * b->tmaps.size(),
@@ -265,17 +258,16 @@ id_status build_items(id_batch* b, int item_mb) {
   return ID_OK;
 }
 
-// The QR jobs of the work-list problems for these output pointers, one per
-// job (in job order).
+// The QR jobs of the work-list problems for these output pointers, the
+// longest first.
 id_status upload_qr_jobs(id_batch* b, int32_t* J, double* P, int32_t* kout) {
   std::vector<QrJob> q;
-  for (const BatchJob& jb : b->jobs) {
-    const int i = jb.prob;
+  for (size_t jq = 0; jq < b->jobs.size(); ++jq) {
+    const int i = b->jobs[jq].prob;
     const id_batch_problem& p = b->prob[i];
     const id_sketch* h = b->h[i];
     QrJob j;
     memset(&j, 0, sizeof(j));
-    j.M = h->d_work;
     j.R = h->d_R;
     j.J = J + b->joff[i];
     j.colpos = h->d_colpos;
@@ -284,8 +276,12 @@ id_status upload_qr_jobs(id_batch* b, int32_t* J, double* P, int32_t* kout) {
     j.rows = p.l;
     j.n = p.n;
     j.k = p.k;
+    j.job = (int32_t)jq;
     q.push_back(j);
   }
+  std::stable_sort(q.begin(), q.end(), [](const QrJob& x, const QrJob& y) {
+    return (double)x.k * x.n * x.rows > (double)y.k * y.n * y.rows;
+  });
   if (q.empty()) return ID_OK;
   const cudaError_t e = cudaMemcpy(b->d_qr, q.data(), sizeof(QrJob) * q.size(),
                                    cudaMemcpyHostToDevice);
@@ -343,11 +339,20 @@ id_status capture(id_batch* b, int32_t* J, double* P, int32_t* kout) {
   if (e != cudaSuccess) s = ID_ERR_CUDA;
   // the work list on the origin stream, the other problems on their branches
   if (s == ID_OK && !b->pers.empty()) {
-    e = cudaMemsetAsync(b->d_counter, 0, sizeof(int) * (1 + b->jobs.size()), b->origin);
+    int kmax = 0, nmax = 0;
+    for (const BatchJob& j : b->jobs) {
+      kmax = std::max(kmax, b->prob[j.prob].k);
+      nmax = std::max(nmax, (int)j.ncols);
+    }
+    const int njobs = (int)b->jobs.size();
+    e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->origin);
     if (e == cudaSuccess)
       e = launch_sketch_batch(b->d_jobs, b->d_tmaps, b->d_items, b->d_order, b->nitems,
-                              b->d_slabs, b->d_counter, b->d_qr, ID_RANK_TOL_FACTOR, b->d_stat,
-                              std::min(b->nsm, b->nitems), kBatchDrainBlocks, b->origin);
+                              b->d_slabs, b->d_counter, b->d_stat, std::min(b->nsm, b->nitems),
+                              kBatchDrainBlocks, b->origin);
+    if (e == cudaSuccess)
+      e = launch_qr_batch(b->d_qr, njobs, b->d_jobs, b->d_items, b->d_slabs, kmax, nmax,
+                          ID_RANK_TOL_FACTOR, b->origin);
     if (e != cudaSuccess) s = ID_ERR_CUDA;
   }
   for (size_t i = 0; i < b->prob.size() && s == ID_OK; ++i)

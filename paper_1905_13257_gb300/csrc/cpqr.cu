@@ -11,11 +11,12 @@
 // from the updated matrix at every step (no downdating) and compared as its
 // square, ties to the lowest column index.
 //
-// n <= 1024 and l <= 64 (cpqr_cluster_kernel): a cluster of 8 CTAs, every column
-// held in the registers of G lanes; one cluster barrier per step.
-// Larger n, or l > 64 rows (cpqr_small_kernel, up to 96 rows): one CTA of 1024
-// threads works in place on a copy of W held row-major in global memory
-// (L2-resident); thread t owns columns t, t + 1024, ...
+// n <= 1024 and l <= 64, or n <= 512 and l <= 96 (cpqr_cluster_kernel, and
+// cpqr_batch_kernel for a batch): a cluster of 8 CTAs, every column held in the
+// registers of G lanes; one cluster barrier per step.
+// Larger n (cpqr_small_kernel): one CTA of 1024 threads works in place on a
+// copy of W held row-major in global memory (L2-resident); thread t owns
+// columns t, t + 1024, ...
 // In both, sums run in a fixed order.
 //
 // Candidates.  With cpos (one int per column) only the columns with
@@ -26,7 +27,10 @@
 #include <cooperative_groups.h>
 #include <float.h>
 
+#include <type_traits>
+
 #include "cta_qr.cuh"
+#include "df.cuh"
 #include "idsk_internal.h"
 
 namespace cg = cooperative_groups;
@@ -55,9 +59,17 @@ constexpr int CL_THREADS = CL_WORKERS + 32;   // and one warp for the step's sca
 // A candidate column: its residual norm as an ordered integer (0: none), its
 // place in the tie order, its index, its rows.
 struct Cand {
-  double col[kLMax];
+  double col[kLMaxW];
   unsigned long long key;
   int ord, j;
+};
+
+// Shared scratch of one QR.
+struct ClusterQr {
+  Cand inbox[2][CL_CTAS];   // every CTA's best candidate, by step parity
+  Cand wbest[CL_WARPS];
+  double fro_w[CL_WARPS], fro_in[CL_CTAS];
+  double gamma, v0, beta;
 };
 
 __device__ __forceinline__ bool nonzero(double x) {   // on the integer units
@@ -87,6 +99,51 @@ __device__ __forceinline__ int best_of_8(const Cand* c, int lane) {
   return (__ffs(__ballot_sync(0xffffffffu, win)) - 1) & 7;
 }
 
+// The matrix of a QR: W itself (row-major) ...
+struct MatrixSrc {
+  const double* M;
+  int64_t ld;
+  template <int G, int RPT>
+  __device__ __forceinline__ void fill(double (&c)[RPT], int g, int j, int rows) const {
+#pragma unroll
+    for (int q = 0; q < RPT; ++q)
+      if (g + G * q < rows) c[q] = M[(int64_t)(g + G * q) * ld + j];
+  }
+};
+// ... or, in a batch, the sum of the work items' FP32 slabs in item order as
+// FP32 pairs (deterministic), four slabs' rows in flight per lane.
+struct SlabSrc {
+  const BatchItem* items;   // the job's
+  const float* slabs;
+  int nitem, lw;
+  template <int G, int RPT>
+  __device__ __forceinline__ void fill(double (&c)[RPT], int g, int j, int rows) const {
+    constexpr int AHEAD = 4;
+    float hi[RPT], lo[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) hi[q] = lo[q] = 0.f;
+    const float* src = slabs + (int64_t)j * lw + g;
+    for (int i0 = 0; i0 < nitem; i0 += AHEAD) {
+      float x[AHEAD][RPT];
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u) {
+        const float* p = src + items[min(i0 + u, nitem - 1)].slab;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) x[u][q] = g + G * q < lw ? p[G * q] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u)
+        if (i0 + u < nitem) {
+#pragma unroll
+          for (int q = 0; q < RPT; ++q) df_add(hi[q], lo[q], x[u][q], 0.f);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < RPT; ++q)
+      if (g + G * q < rows) c[q] = (double)hi[q] + (double)lo[q];
+  }
+};
+
 // Column-pivoted Householder QR of M (rows x n row-major, rows <= 64, n <=
 // 8 * 256 / G) by a cluster of 8 CTAs.  M is only read.
 //
@@ -108,18 +165,19 @@ __device__ __forceinline__ int best_of_8(const Cand* c, int lane) {
 // barriers, every row in every step, 12.9 us a step for any n): n = 512 640 ->
 // 248 us, n = 200 (k = 20, l = 30) 258 -> 86 us, n = 1000 1779 us in one CTA
 // -> 387 us.
-template <int G>
-__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
-    cpqr_cluster_kernel(const double* __restrict__ M, int rows, int n, int64_t ld, int k,
-                        double tol_factor, const int* __restrict__ cpos, double* __restrict__ R,
-                        int* __restrict__ J, int* __restrict__ colpos, int* __restrict__ kout) {
-  constexpr int RPT = kLMax / G;   // rows per lane
+// LM: most rows (64 or 96).  src.fill(c, g, j, rows) loads a lane's rows g, g +
+// G, ... of column j (rows past the last: zero).
+template <int G, int LM, typename Src>
+__device__ __forceinline__ void cluster_qr(const Src& src, int rows, int n, int k,
+                                           double tol_factor,
+                                           const int* __restrict__ cpos, double* __restrict__ R,
+                                           int* __restrict__ J, int* __restrict__ colpos,
+                                           int* __restrict__ kout, ClusterQr& sh) {
+  constexpr int RPT = LM / G;   // rows per lane
   cg::cluster_group cl = cg::this_cluster();
   cl.barrier_arrive();   // waited for before the first write into another CTA
-  __shared__ Cand inbox[2][CL_CTAS];   // every CTA's best candidate, by step parity
-  __shared__ Cand wbest[CL_WARPS];
-  __shared__ double fro_w[CL_WARPS], fro_in[CL_CTAS];
-  __shared__ double sh_gamma, sh_v0, sh_beta;
+  auto& inbox = sh.inbox;
+  auto& wbest = sh.wbest;
   const int rank = (int)cl.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const bool worker = warp < CL_WARPS;
@@ -131,8 +189,8 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
 
   double c[RPT];
 #pragma unroll
-  for (int q = 0; q < RPT; ++q)
-    c[q] = (have && g + G * q < rows) ? M[(int64_t)(g + G * q) * ld + j] : 0.0;
+  for (int q = 0; q < RPT; ++q) c[q] = 0.0;
+  if (have) src.template fill<G>(c, g, j, rows);
   int ord = 0x7fffffff;   // place in the tie order; past the last: never a pivot
   if (have) {
     ord = cpos ? cpos[j] : j;
@@ -159,14 +217,14 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
     double f = ord != 0x7fffffff ? ss : 0.0;
 #pragma unroll
     for (int o = G; o < 32; o <<= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0) fro_w[warp] = f;
+    if (lane == 0) sh.fro_w[warp] = f;
   }
   __syncthreads();
   cl.barrier_wait();
   if (t < CL_CTAS) {
     double f = 0.0;
-    for (int w = 0; w < CL_WARPS; ++w) f += fro_w[w];
-    *cl.map_shared_rank(&fro_in[rank], t) = f;   // read after step 0's cluster barrier
+    for (int w = 0; w < CL_WARPS; ++w) f += sh.fro_w[w];
+    *cl.map_shared_rank(&sh.fro_in[rank], t) = f;   // read after step 0's cluster barrier
   }
   double tol2 = 0.0;
 
@@ -196,10 +254,10 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
     // the CTA's candidate into every CTA's inbox
     {
       const int w = best_of_8(wbest, lane);
-      for (int e = t; e < CL_CTAS * kLMax; e += CL_THREADS) {
-        const int i = e & (kLMax - 1);
+      for (int e = t; e < CL_CTAS * LM; e += CL_THREADS) {
+        const int i = e % LM;
         if (i >= s && i < rows)
-          cl.map_shared_rank(&inbox[b][rank], e / kLMax)->col[i] = wbest[w].col[i];
+          cl.map_shared_rank(&inbox[b][rank], e / LM)->col[i] = wbest[w].col[i];
       }
       if (t < CL_CTAS) {
         Cand* dst = cl.map_shared_rank(&inbox[b][rank], t);
@@ -212,7 +270,7 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
     const Cand& pc = inbox[b][best_of_8(inbox[b], lane)];
     if (s == 0) {
       double f = 0.0;
-      for (int x = 0; x < CL_CTAS; ++x) f += fro_in[x];
+      for (int x = 0; x < CL_CTAS; ++x) f += sh.fro_in[x];
       const double tol = tol_factor * DBL_EPSILON * sqrt(f);
       tol2 = tol * tol;
     }
@@ -225,7 +283,8 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
       const double a0 = pc.col[s];
       const double x0 = s + 1 + lane < rows ? pc.col[s + 1 + lane] : 0.0;
       const double x1 = s + 33 + lane < rows ? pc.col[s + 33 + lane] : 0.0;
-      const bool any = __any_sync(0xffffffffu, nonzero(x0) || nonzero(x1));
+      const double x2 = (LM > 64 && s + 65 + lane < rows) ? pc.col[s + 65 + lane] : 0.0;
+      const bool any = __any_sync(0xffffffffu, nonzero(x0) || nonzero(x1) || nonzero(x2));
       if (lane == 0) {
         double beta = a0, gamma = 0.0, v0 = 0.0;
         if (any) {
@@ -234,9 +293,9 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
           v0 = a0 - beta;
           gamma = 1.0 / (nrm2 + fabs(a0) * nrm);
         }
-        sh_beta = beta;
-        sh_gamma = gamma;
-        sh_v0 = v0;
+        sh.beta = beta;
+        sh.gamma = gamma;
+        sh.v0 = v0;
         if (rank == 0) {
           J[s] = p;
           colpos[p] = s;
@@ -258,8 +317,8 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
     }
     __syncthreads();
     if (busy) {
-      const double v0 = sh_v0;
-      const double w = sh_gamma * (d + v0 * cs);
+      const double v0 = sh.v0;
+      const double w = sh.gamma * (d + v0 * cs);
       ss = 0.0;
 #pragma unroll
       for (int q = 0; q < RPT; ++q) {
@@ -272,12 +331,52 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
       ss = group_sum(ss);
       if (j == p) piv = true;
       if (have && g == 0)
-        R[(int64_t)s * n + j] = j == p ? sh_beta : (piv ? 0.0 : cs - w * v0);
+        R[(int64_t)s * n + j] = j == p ? sh.beta : (piv ? 0.0 : cs - w * v0);
     }
   }
   if (rank == 0) {
     if (t == 0) *kout = s;
     for (int q = s + t; q < k; q += CL_THREADS) J[q] = -1;
+  }
+}
+
+template <int G, int LM>
+__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
+    cpqr_cluster_kernel(const double* __restrict__ M, int rows, int n, int64_t ld, int k,
+                        double tol_factor, const int* __restrict__ cpos, double* __restrict__ R,
+                        int* __restrict__ J, int* __restrict__ colpos, int* __restrict__ kout) {
+  __shared__ ClusterQr sh;
+  cluster_qr<G, LM>(MatrixSrc{M, ld}, rows, n, k, tol_factor, cpos, R, J, colpos, kout, sh);
+}
+
+// The slab sums and pivoted QRs of a batch, one cluster per job (n <= 512): all
+// of them run at once, on up to 8 SMs each.
+__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
+    cpqr_batch_kernel(const QrJob* __restrict__ jobs, const BatchJob* __restrict__ bjobs,
+                      const BatchItem* __restrict__ items, const float* __restrict__ slabs,
+                      double tol_factor) {
+  __shared__ ClusterQr sh;
+  const QrJob q = jobs[blockIdx.x / CL_CTAS];
+  const BatchJob& bj = bjobs[q.job];
+  const SlabSrc src{items + bj.item0, slabs, bj.nitem, w_width(q.rows, false)};
+  const int cols = (q.n + CL_CTAS - 1) / CL_CTAS;
+  auto go = [&](auto g, auto lm) {
+    cluster_qr<decltype(g)::value, decltype(lm)::value>(src, q.rows, q.n, q.k, tol_factor,
+                                                        nullptr, q.R, q.J, q.colpos, q.kout, sh);
+  };
+  using L64 = std::integral_constant<int, 64>;
+  using L96 = std::integral_constant<int, 96>;
+  if (q.rows <= 64) {
+    if (cols <= CL_WORKERS / 16)
+      go(std::integral_constant<int, 16>(), L64());
+    else if (cols <= CL_WORKERS / 8)
+      go(std::integral_constant<int, 8>(), L64());
+    else
+      go(std::integral_constant<int, 4>(), L64());
+  } else if (cols <= CL_WORKERS / 8) {
+    go(std::integral_constant<int, 8>(), L96());
+  } else {
+    go(std::integral_constant<int, 4>(), L96());
   }
 }
 
@@ -307,11 +406,21 @@ __global__ void __launch_bounds__(SP_WARPS * 32) solve_p_kernel(
   solve_p_body(R, J, colpos, kout, k, n, P, blockIdx.x);
 }
 
+__global__ void __launch_bounds__(SP_WARPS * 32) solve_batch_kernel(
+    const QrJob* __restrict__ jobs) {
+  const QrJob q = jobs[blockIdx.y];
+  if ((int)blockIdx.x * SP_WARPS >= q.n) return;
+  solve_p_body(q.R, q.J, q.colpos, q.kout, q.k, q.n, q.P, blockIdx.x);
+}
+
 
 }  // namespace
 
-bool cpqr_cluster_ok(int rows, int64_t n) { return rows <= kLMax && n <= 1024; }
+bool cpqr_cluster_ok(int rows, int64_t n) {
+  return n <= (rows <= kLMax ? 1024 : 512) && rows <= kLMaxW;
+}
 
+// Up to 512 columns for 65 to 96 rows (24 or fewer rows a lane).
 // The cluster form reads W itself; the one-CTA form works in place on a copy
 // of W in `work` (rows x n).  G: the most lanes per column that n columns on 8
 // CTAs of 256 threads allow.
@@ -325,14 +434,15 @@ cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int ro
       kern<<<CL_CTAS, CL_THREADS, 0, st>>>(W, rows, n, ldw, k, tol_factor, cpos, R, J, colpos,
                                            kout);
     };
+    const bool wide = rows > kLMax;
     if (cols <= CL_WORKERS / 16)
-      go(cpqr_cluster_kernel<16>);
+      wide ? go(cpqr_cluster_kernel<16, 96>) : go(cpqr_cluster_kernel<16, 64>);
     else if (cols <= CL_WORKERS / 8)
-      go(cpqr_cluster_kernel<8>);
+      wide ? go(cpqr_cluster_kernel<8, 96>) : go(cpqr_cluster_kernel<8, 64>);
     else if (cols <= CL_WORKERS / 4)
-      go(cpqr_cluster_kernel<4>);
+      wide ? go(cpqr_cluster_kernel<4, 96>) : go(cpqr_cluster_kernel<4, 64>);
     else
-      go(cpqr_cluster_kernel<2>);
+      go(cpqr_cluster_kernel<2, 64>);
   } else {
     const cudaError_t e =
         cudaMemcpy2DAsync(work, sizeof(double) * n, W, sizeof(double) * ldw, sizeof(double) * n,
@@ -341,6 +451,25 @@ cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int ro
     cpqr_small_kernel<<<1, NT, 0, st>>>(work, rows, n, n, k, tol_factor, cpos, R, J, colpos, kout);
   }
   count_launches(1);
+  return cudaGetLastError();
+}
+
+// The QRs of a batch and their solves, in job order (the caller puts the long
+// ones first).
+cudaError_t launch_qr_batch(const QrJob* jobs, int njobs, const BatchJob* bjobs,
+                            const BatchItem* items, const float* slabs, int kmax, int nmax,
+                            double tol_factor, cudaStream_t st) {
+  if (njobs <= 0) return cudaSuccess;
+  cpqr_batch_kernel<<<njobs * CL_CTAS, CL_THREADS, 0, st>>>(jobs, bjobs, items, slabs, tol_factor);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const size_t sm = sizeof(double) * (size_t)kmax * kmax;
+  e = cudaFuncSetAttribute(solve_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sm);
+  if (e != cudaSuccess) return e;
+  solve_batch_kernel<<<dim3((nmax + SP_WARPS - 1) / SP_WARPS, njobs), SP_WARPS * 32, sm, st>>>(
+      jobs);
+  count_launches(2);
   return cudaGetLastError();
 }
 

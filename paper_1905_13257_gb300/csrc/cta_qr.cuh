@@ -1,8 +1,6 @@
-// One-CTA pivoted QR of a small row-major matrix held in global memory and
-// the solve for the interpolation matrix P (Algorithm 4 steps 4-8,
-// transposed).  Used by the pivoted-QR kernels and by the batched sketch
-// kernel, which finishes each matrix of a batch in the CTA that completes its
-// last work item.
+// One-CTA pivoted QR of a small row-major matrix held in global memory (more
+// columns than a cluster's registers hold) and the solve for the interpolation
+// matrix P (Algorithm 4 steps 4-8, transposed).
 #pragma once
 
 #include <float.h>

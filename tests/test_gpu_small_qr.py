@@ -42,6 +42,50 @@ def test_small_qr_forms(n, k, l):
     sk.close()
 
 
+@pytest.mark.parametrize("n,k,l", [(70, 65, 65), (128, 80, 90), (129, 86, 96), (256, 70, 81),
+                                   (257, 66, 96), (512, 80, 90), (513, 30, 70)])
+def test_wide_qr_forms(n, k, l):
+    """65 to 96 rows (FP32 data without Y): the cluster up to 512 columns, one
+    CTA past them."""
+    from paper_1905_13257_gb300 import IdSketch
+    A = gaussian_matrix(1024, n, seed=n + l, dtype=torch.float32, device="cuda")
+    A = A * torch.linspace(0.5, 2.0, n, dtype=torch.float32, device="cuda")
+    sk = IdSketch(1024, n, k, l, seed=3, dtype=torch.float32, want_Y=False)
+    sk.stream_columns(A.T.contiguous().T)
+    W = sk.sketches()[0].cpu().numpy().copy()
+    _check(*sk.factor(), *oracle.column_id(W, k), n)
+    sk.close()
+
+
+def test_batch_qr_forms():
+    """The batch's QRs over their forms in one run: each problem's J and P
+    equal those of one handle (whose W differs in FP32 summation order only,
+    so P within 1e-4 of its scale, J at the oracle's margin)."""
+    from paper_1905_13257_gb300 import IdBatch, IdSketch
+    probs = []
+    for n, k, l in [(64, 10, 20), (128, 64, 64), (129, 20, 30), (300, 40, 50), (512, 50, 60),
+                    (200, 70, 80), (512, 86, 96), (8, 8, 8)]:
+        A = gaussian_matrix(2048, n, seed=n + l, dtype=torch.float32, device="cuda")
+        A = A * torch.linspace(0.5, 2.0, n, dtype=torch.float32, device="cuda")
+        probs.append(dict(A=A.T.contiguous().T, k=k, l=l, seed=n))
+    bt = IdBatch(probs)
+    bt.run()
+    out = bt.wait()
+    for p, (J, P, kout) in zip(probs, out):
+        n = p["A"].shape[1]
+        sk = IdSketch(2048, n, p["k"], p["l"], seed=p["seed"], want_Y=False)
+        sk.stream_columns(p["A"])
+        J1, P1, k1 = sk.factor()
+        margin = oracle.column_id(sk.sketches()[0].cpu().numpy(), p["k"])[3]
+        assert kout == k1 == p["k"]
+        assert_valid_skeleton(J.cpu().numpy(), P.cpu().numpy(), kout, n)
+        if margin >= MARGIN:
+            assert torch.equal(J, J1)
+            assert (P - P1).abs().max().item() <= 1e-4 * max(1.0, P1.abs().max().item())
+        sk.close()
+    bt.close()
+
+
 @pytest.mark.parametrize("n,ncand,k,l", [(40, 12, 6, 16), (300, 90, 25, 40), (512, 100, 50, 60),
                                          (1100, 64, 20, 30)])
 def test_restricted_qr_forms(n, ncand, k, l):
