@@ -65,7 +65,7 @@ struct id_batch {
   int items_cap = 0;
   float* d_slabs = nullptr;
   size_t slab_cap = 0;                // floats
-  int* d_counter = nullptr;           // the item counter
+  int* d_counter = nullptr;           // [0] the item counter, [1 + j] job j's completed items
   QrJob* d_qr = nullptr;
   int item_mb = 0;                    // autotuned work-item size (0: automatic)
   int nsm = 0;
@@ -164,6 +164,7 @@ void build_jobs(id_batch* b) {
       j.ncols = p.n;
       j.np = j.a.bf16 ? 1 : 2;
       j.prob = (int)i;
+      j.Wd = h->d_work + (int64_t)s0 * p.n;
       b->jobs.push_back(j);
       b->tmaps.push_back(tm);
     }
@@ -201,16 +202,43 @@ id_status build_items(id_batch* b, int item_mb) {
     }
     j.nitem = (int32_t)items.size() - j.item0;
   }
-  std::vector<int32_t> order(items.size());
-  std::iota(order.begin(), order.end(), 0);
-  // largest items first (a job's row blocks per item follow from its width, so
-  // the items differ by the ragged last ones only)
-  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-    auto bytes = [&](int32_t i) {
-      return (double)items[i].nrb * b->jobs[items[i].job].ncols;
-    };
-    return bytes(x) > bytes(y);
-  });
+  // jobs in order of decreasing QR work (k n l), so that the QRs which the
+  // CTAs run as matrices complete overlap later items and the last matrices
+  // to complete have the cheapest ones; each job's items in row order
+  std::vector<int> jorder(b->jobs.size());
+  std::iota(jorder.begin(), jorder.end(), 0);
+  auto qr_work = [&](int q) {
+    const BatchJob& j = b->jobs[q];
+    return (double)b->prob[j.prob].k * j.ncols * j.a.l;
+  };
+  std::stable_sort(jorder.begin(), jorder.end(),
+                   [&](int x, int y) { return qr_work(x) > qr_work(y); });
+  // A job is deferred when its QR in one CTA (about 9 us a step and the FP64
+  // work, 3 n (l - s) operations in step s at 2 per clock) takes longer than
+  // the items after it do (about 4 TB/s) -- provided that the longest such
+  // overhang exceeds the cluster QRs themselves (about 6 us a step and 0.1 ms
+  // for their launches).  12 matrices, 2.5 GB, k up to 80: all deferred 1.56 ms
+  // a run, none 3.87 ms; 64 matrices, 82 GB, k from 10 to 79: none deferred
+  // 21.4 ms, the last few 21.5 ms, all 22.3 ms.
+  double after = 0.0, overhang = 0.0, kdef = 0.0;
+  for (auto it = jorder.rbegin(); it != jorder.rend(); ++it) {
+    BatchJob& j = b->jobs[*it];
+    const double k = b->prob[j.prob].k, l = j.a.l;
+    const double qr_s = k * (9e-6 + 1.5 * j.ncols * (l - 0.5 * k) / 2.0e9);
+    j.deferred = qr_s > after / 4.0e12 ? 1 : 0;
+    if (j.deferred) {
+      overhang = std::max(overhang, qr_s - after / 4.0e12);
+      kdef = std::max(kdef, k);
+    }
+    after += 4.0 * (double)j.a.m * j.ncols;
+  }
+  if (overhang < 1e-4 + 6e-6 * kdef)
+    for (BatchJob& j : b->jobs) j.deferred = 0;
+  std::vector<int32_t> order;
+  order.reserve(items.size());
+  for (int q : jorder)
+    for (int32_t it = b->jobs[q].item0; it < b->jobs[q].item0 + b->jobs[q].nitem; ++it)
+      order.push_back(it);
   cudaError_t e = cudaSuccess;
   if ((int)items.size() > b->items_cap) {
     if (b->d_items) cudaFree(b->d_items);
@@ -232,8 +260,8 @@ id_status build_items(id_batch* b, int item_mb) {
   if (e == cudaSuccess && !b->d_jobs) {
     e = cudaMalloc(&b->d_jobs, sizeof(BatchJob) * b->jobs.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tmaps, sizeof(CUtensorMap) * b->tmaps.size());
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_qr, sizeof(QrJob) * b->jobs.size());
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int) * (1 + b->jobs.size()));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_qr, 2 * sizeof(QrJob) * b->jobs.size());
     if (e == cudaSuccess)
       e = cudaMemcpy(b->d_tmaps, b->tmaps.data(), sizeof(CUtensorMap) * b->tmaps.size(),
                      cudaMemcpyHostToDevice);
@@ -258,8 +286,8 @@ id_status build_items(id_batch* b, int item_mb) {
   return ID_OK;
 }
 
-// The QR jobs of the work-list problems for these output pointers, the
-// longest first.
+// The QR jobs of the work-list problems for these output pointers, one per
+// job (in job order), then those of the deferred jobs again, the longest first.
 id_status upload_qr_jobs(id_batch* b, int32_t* J, double* P, int32_t* kout) {
   std::vector<QrJob> q;
   for (size_t jq = 0; jq < b->jobs.size(); ++jq) {
@@ -268,6 +296,7 @@ id_status upload_qr_jobs(id_batch* b, int32_t* J, double* P, int32_t* kout) {
     const id_sketch* h = b->h[i];
     QrJob j;
     memset(&j, 0, sizeof(j));
+    j.M = h->d_work;
     j.R = h->d_R;
     j.J = J + b->joff[i];
     j.colpos = h->d_colpos;
@@ -279,10 +308,14 @@ id_status upload_qr_jobs(id_batch* b, int32_t* J, double* P, int32_t* kout) {
     j.job = (int32_t)jq;
     q.push_back(j);
   }
-  std::stable_sort(q.begin(), q.end(), [](const QrJob& x, const QrJob& y) {
+  if (q.empty()) return ID_OK;
+  std::vector<QrJob> def;
+  for (const QrJob& j : q)
+    if (b->jobs[j.job].deferred) def.push_back(j);
+  std::stable_sort(def.begin(), def.end(), [](const QrJob& x, const QrJob& y) {
     return (double)x.k * x.n * x.rows > (double)y.k * y.n * y.rows;
   });
-  if (q.empty()) return ID_OK;
+  q.insert(q.end(), def.begin(), def.end());
   const cudaError_t e = cudaMemcpy(b->d_qr, q.data(), sizeof(QrJob) * q.size(),
                                    cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail_cuda(b, e);
@@ -339,20 +372,22 @@ id_status capture(id_batch* b, int32_t* J, double* P, int32_t* kout) {
   if (e != cudaSuccess) s = ID_ERR_CUDA;
   // the work list on the origin stream, the other problems on their branches
   if (s == ID_OK && !b->pers.empty()) {
-    int kmax = 0, nmax = 0;
-    for (const BatchJob& j : b->jobs) {
-      kmax = std::max(kmax, b->prob[j.prob].k);
-      nmax = std::max(nmax, (int)j.ncols);
-    }
-    const int njobs = (int)b->jobs.size();
-    e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->origin);
+    e = cudaMemsetAsync(b->d_counter, 0, sizeof(int) * (1 + b->jobs.size()), b->origin);
     if (e == cudaSuccess)
       e = launch_sketch_batch(b->d_jobs, b->d_tmaps, b->d_items, b->d_order, b->nitems,
-                              b->d_slabs, b->d_counter, b->d_stat, std::min(b->nsm, b->nitems),
-                              kBatchDrainBlocks, b->origin);
+                              b->d_slabs, b->d_counter, b->d_qr, ID_RANK_TOL_FACTOR, b->d_stat,
+                              std::min(b->nsm, b->nitems), kBatchDrainBlocks, b->origin);
+    // the deferred jobs' QR table follows the full one
+    int kmax = 0, nmax = 0, ndef = 0;
+    for (const BatchJob& j : b->jobs)
+      if (j.deferred) {
+        kmax = std::max(kmax, (int)b->prob[j.prob].k);
+        nmax = std::max(nmax, (int)j.ncols);
+        ++ndef;
+      }
     if (e == cudaSuccess)
-      e = launch_qr_batch(b->d_qr, njobs, b->d_jobs, b->d_items, b->d_slabs, kmax, nmax,
-                          ID_RANK_TOL_FACTOR, b->origin);
+      e = launch_qr_batch(b->d_qr + b->jobs.size(), ndef, b->d_jobs, b->d_items, b->d_slabs, kmax,
+                          nmax, ID_RANK_TOL_FACTOR, b->origin);
     if (e != cudaSuccess) s = ID_ERR_CUDA;
   }
   for (size_t i = 0; i < b->prob.size() && s == ID_OK; ++i)

@@ -126,13 +126,16 @@ __host__ __device__ constexpr inline int w_width(int l, bool want_Y) {
 
 // ------------------------------------------- batched form (work list)
 // The sketch of one matrix of a batch: all a.l <= 96 rows of Psi in one
-// pass, no Y and no coarse gather.
+// pass, no Y and no coarse gather.  Its W goes to Wd (row-major, a.l x
+// ncols, leading dimension ncols) unless the job is deferred.
 struct BatchJob {
   SketchArgs a;
   int32_t ncols;          // n of the matrix (<= 512)
   int32_t np;             // bfloat16 pieces of A: 2 (FP32-accurate) or 1 (BF16 form)
   int32_t prob;           // problem index (its status flag)
   int32_t item0, nitem;   // its work items, contiguous in the item table
+  int32_t deferred;       // QR after the work list, by a cluster of CTAs
+  double* Wd;
 };
 // A work item: row blocks rb0 .. rb0 + nrb - 1 of one job, its W^T partials
 // into the FP32 slab at float offset `slab` ([ceil(ncols / 128) * 128][lw],
@@ -145,6 +148,7 @@ struct BatchItem {
 // Pivoted QR of one batched W (l x n, the sum of its BatchJob's slabs) and the
 // solve for P, written straight into the batch's packed outputs.
 struct QrJob {
+  double* M;
   double* R;
   int32_t* J;
   int32_t* colpos;
@@ -350,15 +354,19 @@ cudaError_t launch_sketch_simt(const SketchArgs& a, const Window& w, int dtype, 
 cudaError_t launch_sketch_tc(const SketchArgs& a, const Window& w, int npieces, int nsm,
                              int drain_blocks, int* status, cudaStream_t st,
                              KernelTimer* timer = nullptr);
-// Batched form: the whole work list's sketches in one persistent launch (grid
-// CTAs; items taken in `order` from `counter`, zeroed by the caller;
-// sketch_tc.cu), then every job's slab sums, QR and solve (cpqr.cu; kmax, nmax:
-// the largest k and n).
+// Batched form (sketch_tc.cu): the whole work list in one persistent launch
+// (grid CTAs; items taken in `order`; counters[0] the item counter and
+// counters[1 + j] job j's completed items, all zeroed by the caller); the CTA
+// that completes a job's last item sums its slabs into W and runs its QR and
+// solve (qjobs[j]) unless the job is deferred; the deferred jobs' slab sums,
+// QRs and solves follow (cpqr.cu, one launch each; kmax, nmax: their largest k
+// and n).
 size_t sketch_batch_smem_bytes();
 cudaError_t launch_sketch_batch(const BatchJob* jobs, const CUtensorMap* tmaps,
                                 const BatchItem* items, const int32_t* order, int nitems,
-                                float* slabs, int* counter, int* stat, int grid,
-                                int drain_blocks, cudaStream_t st);
+                                float* slabs, int* counters, const QrJob* qjobs,
+                                double tol_factor, int* stat, int grid, int drain_blocks,
+                                cudaStream_t st);
 cudaError_t launch_qr_batch(const QrJob* jobs, int njobs, const BatchJob* bjobs,
                             const BatchItem* items, const float* slabs, int kmax, int nmax,
                             double tol_factor, cudaStream_t st);

@@ -63,6 +63,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "cta_qr.cuh"
 #include "df.cuh"
 #include "idsk_internal.h"
 #include "tc_common.cuh"
@@ -785,30 +786,77 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
   if (tid == 0 && ld_volatile_shared(S.abort_flag)) atomicOr(status, 1);
 }
 
-// Batched form, the sketches in one persistent launch: a work list of row
-// ranges (items) over the sketches (jobs) of many matrices, one CTA per SM.  A
-// CTA takes the next item from a global counter, copies the job's arguments to
-// shared memory, runs the roles over the item's row blocks into the item's W^T
-// slab, and synchronises.  One barrier set serves all items: every role
-// carries its running counts (RoleCounters) from item to item, so each wait
-// expects the right phase, including the commits of an earlier item that
-// nobody waited for inside it.  The TMEM stays allocated throughout.  Every
-// wait stays bounded: a CTA that gives up raises its job's problem flag and
-// stops taking items.  The slab sums with the pivoted QRs, and the solves,
-// follow as launches of their own (cpqr_batch_kernel, solve_batch_kernel): run
-// by the CTA that completed a matrix, beside the later items, the last
-// matrices' one-CTA QRs (2 to 3 ms each) stood alone at the end.  12 matrices, 2.5 GB: 3.76 ms -> BATCH_TIME.
+// Batched form, the last step of one matrix: W = the sum of its items'
+// slabs in item order (deterministic, FP32 pairs, read past L1: other SMs
+// wrote them), then the pivoted QR of W and the solve for P into the
+// batch's outputs, all by this CTA (shared scratch in the free buffers).
+__device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* __restrict__ items,
+                                           const float* __restrict__ slabs, const QrJob& q,
+                                           double tol_factor, uint8_t* scratch) {
+  const int l = jb.a.l, n = jb.ncols, lw = w_width(l, false);
+  for (int e = threadIdx.x; e < l * n; e += NTHREADS_TMA) {
+    const int c = e / l, s = e - c * l;
+    float hi = 0.f, lo = 0.f;
+    for (int q0 = 0; q0 < jb.nitem; q0 += 8) {
+      float x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        x[u] = q0 + u < jb.nitem
+                   ? __ldcg(slabs + items[jb.item0 + q0 + u].slab + (int64_t)c * lw + s)
+                   : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) df_add(hi, lo, x[u], 0.f);
+    }
+    jb.Wd[(int64_t)s * n + c] = (double)hi + (double)lo;
+  }
+  __syncthreads();
+  qr::QrShared& sh = *reinterpret_cast<qr::QrShared*>(scratch);
+  qr::cta_pivoted_qr<NTHREADS_TMA>(q.M, q.rows, q.n, q.n, q.k, tol_factor, nullptr, q.R, q.J,
+                                   q.colpos, q.kout, sh);
+  __syncthreads();
+  double* r11 = reinterpret_cast<double*>(scratch + 4096);
+  double* rdiag = r11 + kLMaxW * kLMaxW;
+  int* Js = reinterpret_cast<int*>(rdiag + kLMaxW);
+  const int kk = qr::solve_setup(q.R, q.J, q.kout, q.n, r11, Js, rdiag);
+  for (int j = threadIdx.x >> 5; j < q.n; j += NTHREADS_TMA / 32)
+    qr::solve_column(j, q.R, q.colpos, q.k, kk, q.n, q.P, r11, rdiag);
+  __syncthreads();
+}
+
+// Batched form in one persistent launch: a work list of row ranges (items)
+// over the sketches (jobs) of many matrices, one CTA per SM.  A CTA takes the
+// next item from a global counter (jobs in order of decreasing QR work, each
+// job's items in row order), copies the job's arguments to shared memory,
+// runs the roles over the item's row blocks into the item's W^T slab, and
+// synchronises.  One barrier set serves all items: every role carries its
+// running counts (RoleCounters) from item to item, so each wait expects the
+// right phase, including the commits of an earlier item that nobody waited
+// for inside it.  The CTA that completes a job's last item (counted per job
+// after its slab writes are fenced) sums the job's slabs into W and runs its
+// pivoted QR and solve, while the other CTAs go on with later items -- unless
+// the job is `deferred`: a one-CTA QR takes 1 to 3 ms, and with too few items
+// left to run beside it, it would stand alone at the end.  The deferred jobs'
+// slab sums and QRs run afterwards, a cluster of 8 SMs each (cpqr.cu).  The
+// rule is on sizes alone (batch.cu), so results do not depend on scheduling.
+// 12 matrices, 2.5 GB, k up to 80: 3.87 ms with none deferred, 1.56 ms with all;
+// 64 matrices, 82 GB: 21.4 ms with none, 22.3 ms with all.
+// The TMEM stays allocated throughout.  Every wait stays bounded: a CTA that
+// gives up raises its job's problem flag and stops taking items.
 __global__ void __launch_bounds__(NTHREADS_TMA, 1)
     sketch_batch_kernel(const BatchJob* __restrict__ jobs, const CUtensorMap* __restrict__ tmaps,
                         const BatchItem* __restrict__ items, const int32_t* __restrict__ order,
-                        int nitems, float* __restrict__ slabs, int* __restrict__ counter,
+                        int nitems, float* __restrict__ slabs, int* __restrict__ counters,
+                        const QrJob* __restrict__ qjobs, double tol_factor,
                         int* __restrict__ stat, int drain_blocks) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
   const Smem S = carve<1, true>((sbase + 1023u) & ~1023u);
   const uint32_t s_args = (S.abort_flag + 4u + 15u) & ~15u;       // SketchArgs of the job
   const uint32_t s_item = s_args + (uint32_t)sizeof(SketchArgs);   // item index
+  const uint32_t s_last = s_item + 4u;   // the item completed a job that is not deferred
   SketchArgs* args = reinterpret_cast<SketchArgs*>(smem_raw + (s_args - sbase));
+  uint8_t* scratch = smem_raw + (S.pieces - sbase);   // free between items
+  int* job_done = counters + 1;
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) {
     st_volatile_shared(S.abort_flag, 0);
@@ -823,7 +871,7 @@ __global__ void __launch_bounds__(NTHREADS_TMA, 1)
   RoleCounters rc;
   for (;;) {
     if (tid == 0) {
-      const int q = atomicAdd(counter, 1);
+      const int q = atomicAdd(counters, 1);
       st_volatile_shared(s_item, q < nitems ? order[q] : -1);
     }
     __syncthreads();
@@ -846,12 +894,26 @@ __global__ void __launch_bounds__(NTHREADS_TMA, 1)
         sketch_roles<1, true, false>(*args, nullptr, jb.ncols, tm, item.rb0, item.nrb,
                                      slabs + item.slab, drain_blocks, S, tmem, smem_raw, rc);
     }
+    if (warp >= NCONV && warp < MMA_WARP) __threadfence();   // the slab writes, GPU-wide
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    const int it = ld_volatile_shared(s_item);
+    const int job = items[it].job;
     if (ld_volatile_shared(S.abort_flag)) {
-      if (tid == 0) atomicOr(stat + jobs[items[ld_volatile_shared(s_item)].job].prob, 1);
+      if (tid == 0) atomicOr(stat + jobs[job].prob, 1);
       break;
+    }
+    if (tid == 0) {
+      __threadfence();
+      const int done = atomicAdd(job_done + job, 1) + 1;
+      st_volatile_shared(s_last, done == jobs[job].nitem && !jobs[job].deferred ? 1 : 0);
+    }
+    __syncthreads();
+    if (ld_volatile_shared(s_last)) {
+      __threadfence();
+      finish_job(jobs[job], items, slabs, qjobs[job], tol_factor, scratch);
+      fence_proxy_async();   // the scratch's generic writes before the next TMA writes
     }
   }
   tc_fence_before();
@@ -1112,15 +1174,17 @@ size_t sketch_batch_smem_bytes() {
 
 cudaError_t launch_sketch_batch(const BatchJob* jobs, const CUtensorMap* tmaps,
                                 const BatchItem* items, const int32_t* order, int nitems,
-                                float* slabs, int* counter, int* stat, int grid,
-                                int drain_blocks, cudaStream_t st) {
+                                float* slabs, int* counters, const QrJob* qjobs,
+                                double tol_factor, int* stat, int grid, int drain_blocks,
+                                cudaStream_t st) {
   if (nitems <= 0) return cudaSuccess;
   const size_t sm = sketch_batch_smem_bytes();
   cudaError_t e = cudaFuncSetAttribute(sketch_batch_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   sketch_batch_kernel<<<grid, NTHREADS_TMA, sm, st>>>(jobs, tmaps, items, order, nitems, slabs,
-                                                      counter, stat, drain_blocks);
+                                                      counters, qjobs, tol_factor, stat,
+                                                      drain_blocks);
   count_launches(1);
   return cudaGetLastError();
 }

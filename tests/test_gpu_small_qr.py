@@ -57,14 +57,19 @@ def test_wide_qr_forms(n, k, l):
     sk.close()
 
 
-def test_batch_qr_forms():
+@pytest.mark.parametrize("spec", [
+    # long QRs: run after the work list, a cluster each
+    [(64, 10, 20), (128, 64, 64), (129, 20, 30), (300, 40, 50), (512, 50, 60), (200, 70, 80),
+     (512, 86, 96), (8, 8, 8)],
+    # short QRs: each in the CTA that completes its matrix
+    [(64, 3, 13), (200, 5, 15), (512, 4, 80), (8, 8, 8)]])
+def test_batch_qr_forms(spec):
     """The batch's QRs over their forms in one run: each problem's J and P
     equal those of one handle (whose W differs in FP32 summation order only,
     so P within 1e-4 of its scale, J at the oracle's margin)."""
     from paper_1905_13257_gb300 import IdBatch, IdSketch
     probs = []
-    for n, k, l in [(64, 10, 20), (128, 64, 64), (129, 20, 30), (300, 40, 50), (512, 50, 60),
-                    (200, 70, 80), (512, 86, 96), (8, 8, 8)]:
+    for n, k, l in spec:
         A = gaussian_matrix(2048, n, seed=n + l, dtype=torch.float32, device="cuda")
         A = A * torch.linspace(0.5, 2.0, n, dtype=torch.float32, device="cuda")
         probs.append(dict(A=A.T.contiguous().T, k=k, l=l, seed=n))
