@@ -102,11 +102,9 @@ typedef struct id_sketch id_sketch;   /* opaque, library-owned */
  * cuda_stream may be NULL (legacy default stream).
  * Sketch width: l <= 64 for every form.  FP32 data without Y may take
  * 64 < l <= 96 (k up to 86 at p = 10): the tensor-core sketch then forms W
- * in one pass with 96-wide accumulators when the window is one buffer with
- * 16-byte aligned columns, else in passes of 60 rows of Psi (one more read
- * of the window per pass); the pivoted QR and the solve take the wider W,
- * and the coarse-grid QR, the error pass and the single-pass ID keep
- * k <= 64.
+ * in one pass with 96-wide accumulators; the pivoted QR and the solve take
+ * the wider W, and the coarse-grid QR, the error pass and the single-pass ID
+ * keep k <= 64.
  * Errors: ID_ERR_INVALID_ARG for an inconsistent config (m <= 0, n_max <= 0,
  * k < 1, k > l, l > 96, grid/ncomp not matching m when want_coarse, a coarse
  * stride < 1, reserved fields != 0), ID_ERR_UNSUPPORTED (l > 64 with FP64

@@ -148,7 +148,6 @@ void build_jobs(id_batch* b) {
     b->pers.push_back((int)i);
     b->in_pers[i] = 1;
     {   // all l <= 96 sketch rows in one pass (no Y)
-      const int s0 = 0;
       BatchJob j;
       memset(&j, 0, sizeof(j));
       j.a.m = p.m;
@@ -160,11 +159,10 @@ void build_jobs(id_batch* b) {
       j.a.omega = h->d_omega;
       j.a.ldw = p.n;
       j.a.bf16 = p.prec == ID_SKETCH_BF16 ? 1 : 0;
-      j.a.s0 = s0;
       j.ncols = p.n;
       j.np = j.a.bf16 ? 1 : 2;
       j.prob = (int)i;
-      j.Wd = h->d_work + (int64_t)s0 * p.n;
+      j.Wd = h->d_work;
       b->jobs.push_back(j);
       b->tmaps.push_back(tm);
     }

@@ -14,11 +14,9 @@ namespace idsk {
 // ------------------------------------------------------------------ limits
 constexpr int kLMax = 64;             // sketch width l (padded to 16 on device)
 // Wider sketches, l <= kLMaxW (so k <= 86 at l = k + 10): FP32 data on the
-// tensor-core sketch without Y, in passes of at most kPassRows rows of Psi
-// (one more read of each window per pass); the one-CTA pivoted QR and the
-// solve take up to kLMaxW rows and pivots.  Everything else keeps k, l <= 64.
+// tensor-core sketch without Y; the pivoted QR of W and the solve take up to
+// kLMaxW rows and pivots.  Everything else keeps k, l <= 64.
 constexpr int kLMaxW = 96;
-constexpr int kPassRows = 60;         // a multiple of 10: Psi's counter blocks
 constexpr int kMaxSegs = 64;          // column segments per sketch launch
 constexpr int kSimtWindowMax = 320;   // columns per SIMT sketch launch at most
 constexpr int kTcMaxTiles = 4;        // 128-column tiles per tensor-core launch (TMEM budget)
@@ -114,7 +112,6 @@ struct SketchArgs {
   const int64_t* crow;  // tensor-core path: fine row of each coarse row (the A_c copy)
   const float* colscale;   // FP8 form: 2^e_c of each column of the window (window column 0 first)
   int32_t fp8;             // FP8-E4M3 form (tensor-core path, one bfloat16 piece)
-  int32_t s0;           // first row of Psi drawn by this launch (a multiple of 10)
 };
 
 // Width of the tensor-core sketch's W^T accumulators and partial slabs: 64

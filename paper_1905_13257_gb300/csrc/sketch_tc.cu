@@ -31,10 +31,9 @@
 //
 // Warp roles (one CTA per SM, persistent over a contiguous range of row
 // blocks):
-//   warps 0-7    converters: load A with 128-bit coalesced loads in half
-//                tiles (two register buffers: one half tile in flight),
-//                split into pieces, store them to the swizzled piece buffer
-//                (double-buffered)
+//   warps 0-7    converters: read A from the ring of raw boxes, split it into
+//                pieces and fill two single-piece slots in turn, so that the
+//                MMAs of one piece overlap the conversion of the other
 //   warps 8-11   epilogue: draw Psi for upcoming row blocks (counter
 //                generator), drain Y to global memory, flush W^T partials
 //                into a per-CTA FP32 slab in L2 (one 128-column tile at a
@@ -42,12 +41,16 @@
 //                is handed back to the MMAs as soon as it is in registers,
 //                before its reductions)
 //   warp 12      TMEM allocation and the single-thread tcgen05.mma issue
-//   warp 13      (TMA form: a single-segment window with 16-byte aligned
-//                columns) streams raw FP32 boxes of 128 rows x 32 columns
-//                through an NST-stage shared-memory ring; the converters
-//                then read A from the ring and fill two single-piece slots
-//                in turn, so that the MMAs of one piece overlap the
-//                conversion of the other
+//   warp 13      producer: streams raw FP32 boxes of 128 rows x 32 columns
+//                through an NST-stage shared-memory ring, by a tensor map
+//                where the window is one buffer, else column by column with
+//                16-byte asynchronous copies.  (Windows of several buffers
+//                were read by the converters themselves before, 32 KB in
+//                flight per SM: 589,824 x 512 in 16 buffers with Y took 791
+//                us; with a 512-byte bulk copy per column and box, whose lanes
+//                issue one after the other, 661 us; with these copies by one
+//                warp 448 us, by three 408 us; the tensor map's feed of the
+//                same bytes in one buffer would take about 310 us.)
 // At most 4 warps per SM sub-partition, so a thread may hold up to 128
 // registers.
 // Every mbarrier wait is bounded: on timeout the CTA raises an abort flag,
@@ -80,10 +83,17 @@ constexpr int TCOLS = 128;              // columns per tile
 constexpr int NCONV = 8;                // converter warps
 constexpr int NEPI = 4;                 // epilogue warps
 constexpr int MMA_WARP = NCONV + NEPI;  // 12
-constexpr int NTHREADS = (NCONV + NEPI + 1) * 32;
-constexpr int PROD_WARP = MMA_WARP + 1;   // TMA producer (TMA form only)
-constexpr int NTHREADS_TMA = NTHREADS + 32;
+constexpr int PROD_WARP = MMA_WARP + 1;   // the producer of raw boxes
+constexpr int NTHREADS = (PROD_WARP + 1) * 32;
+constexpr int NPROD = 3;                  // producers of FEED_COLUMNS, boxes in turn
 constexpr int NST = 4;                    // raw FP32 stages of 128 rows x 32 columns
+// How the producer reads A: boxes of a tensor map (a window that is one
+// buffer), or 16-byte asynchronous copies, a column per warp instruction
+// (columns anywhere, each on a 16-byte boundary: a window of several buffers).
+constexpr int FEED_TENSOR = 1, FEED_COLUMNS = 2;
+constexpr int feed_threads(int feed) {
+  return NTHREADS + (feed == FEED_COLUMNS ? 32 * (NPROD - 1) : 0);
+}
 constexpr uint32_t RAW_BYTES = TR * 32 * 4;   // 16 KB
 constexpr int LP = 64;                  // padded sketch width: N of both products
 constexpr uint32_t PIECE_BYTES = TR * TCOLS * 2;     // 32 KB
@@ -115,8 +125,8 @@ enum { B_FULL0 = 0, B_FULL1, B_FREE0, B_FREE1, B_PSIF0, B_PSIE0 = B_PSIF0 + 4,
        B_DONE = B_WE0 + kTcMaxTiles, B_RF0, B_RE0 = B_RF0 + NST, NBAR = B_RE0 + NST };
 
 struct Smem {
-  uint32_t pieces;   // [2 buffers][NP][PIECE_BYTES] (TMA form: [2 slots][PIECE_BYTES])
-  uint32_t raw;      // TMA form: [NST][RAW_BYTES]
+  uint32_t pieces;   // [2 slots][PIECE_BYTES]
+  uint32_t raw;      // [NST][RAW_BYTES]
   uint32_t omega;    // [kTcMaxTiles][OMEGA_TILE_BYTES]
   uint32_t psi;      // [2][PSI_BYTES]
   uint32_t bars;     // NBAR x 8 bytes
@@ -157,21 +167,6 @@ __device__ __forceinline__ const float* column_ptr(const Window& w, int c) {
   return nullptr;
 }
 
-// The loaded value of column c, rows r0..r0+3, with out-of-range entries zero
-// (ragged last row block: the valid rows are read here, element by element).
-__device__ __forceinline__ float4 split_source(const SketchArgs& a, const Window& w, int64_t r0,
-                                               int c, float4 x) {
-  if (r0 + 3 < a.m && c < w.ncols) return x;
-  float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (c < w.ncols && r0 < a.m) {
-    const float* p = column_ptr(w, c) + r0;
-    y.x = p[0];
-    if (r0 + 1 < a.m) y.y = p[1];
-    if (r0 + 2 < a.m) y.z = p[2];
-  }
-  return y;
-}
-
 // FP8 form: two values rounded to the nearest FP8-E4M3 value, ties to even,
 // saturating at +-448 (the hardware conversion), and widened back exactly
 // through half precision (E4M3 values are exact in half and in bfloat16);
@@ -205,7 +200,7 @@ __device__ __forceinline__ void psi_row(const SketchArgs& a, int64_t r, int rl, 
   for (int sb = 0; sb < ngroups; ++sb) {
     float g[10];
     if (r < a.m) {
-      gauss10((uint64_t)r, (uint32_t)(sb + a.s0 / 10), kStreamPsi, a.k0, a.k1, a.table, g);
+      gauss10((uint64_t)r, (uint32_t)sb, kStreamPsi, a.k0, a.k1, a.table, g);
     } else {
 #pragma unroll
       for (int f = 0; f < 10; ++f) g[f] = 0.f;
@@ -219,25 +214,24 @@ __device__ __forceinline__ void psi_row(const SketchArgs& a, int64_t r, int rl, 
   }
 }
 
-// Shared-memory carve-up (1024-byte aligned base).  The batched kernel uses
-// the TMA form's layout and keeps its current job's arguments after the
-// abort flag.
-template <int NP, bool TMA>
+// Shared-memory carve-up (1024-byte aligned base).  The batched kernel keeps its
+// current job's arguments after the abort flag.
 __device__ __forceinline__ Smem carve(uint32_t base) {
   Smem S;
   S.pieces = base;
-  S.omega = S.pieces + (TMA ? 2u : 2u * NP) * PIECE_BYTES;
+  S.omega = S.pieces + 2u * PIECE_BYTES;
   S.psi = S.omega + kTcMaxTiles * OMEGA_TILE_BYTES;
   S.raw = S.psi + 2u * PSI_BYTES;
-  S.bars = S.raw + (TMA ? NST * RAW_BYTES : 0u);
+  S.bars = S.raw + NST * RAW_BYTES;
   S.tmem_slot = S.bars + NBAR * 8u;
   S.abort_flag = S.tmem_slot + 4u;
   return S;
 }
 
 // The CTA's barrier set (thread 0, once per kernel).
-template <bool TMA>
-__device__ __forceinline__ void init_bars(const Smem& S) {
+// box_arrivals: the producer's arrivals per raw box (1 with a transaction count,
+// or one per lane).
+__device__ __forceinline__ void init_bars(const Smem& S, int box_arrivals) {
   auto bar = [&](int i) { return S.bars + 8u * (uint32_t)i; };
   mbar_init(bar(B_FULL0), NCONV);
   mbar_init(bar(B_FULL1), NCONV);
@@ -256,11 +250,9 @@ __device__ __forceinline__ void init_bars(const Smem& S) {
     mbar_init(bar(B_WE0 + ct), NEPI);
   }
   mbar_init(bar(B_DONE), 1);
-  if (TMA) {
-    for (int st = 0; st < NST; ++st) {
-      mbar_init(bar(B_RF0 + st), 1);
-      mbar_init(bar(B_RE0 + st), NCONV);
-    }
+  for (int st = 0; st < NST; ++st) {
+    mbar_init(bar(B_RF0 + st), box_arrivals);
+    mbar_init(bar(B_RE0 + st), NCONV);
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -271,9 +263,8 @@ __device__ __forceinline__ void init_bars(const Smem& S) {
 // at zero).  A thread keeps only its own role's counts.
 struct RoleCounters {
   int g = 0;           // row blocks (epilogue, MMA issuer)
-  int u = 0;           // bfloat16 piece units (TMA converters, MMA issuer)
-  int t = 0;           // tiles (register-form converters and MMA issuer)
-  int box = 0;         // raw TMA boxes (TMA converters, producer)
+  int u = 0;           // bfloat16 piece units (converters, MMA issuer)
+  int box = 0;         // raw boxes (converters, producer)
   int done = 0;        // completed ranges (MMA issuer: phase of B_DONE)
   uint32_t wpar = 0;   // per W^T tile: parity of its flushes (epilogue, MMA issuer)
   uint32_t wpend = 0;  // MMA issuer: tiles handed to the epilogue, not yet read back
@@ -282,9 +273,9 @@ struct RoleCounters {
 // The roles of one CTA over row blocks rb_begin .. rb_begin + nloc - 1 of
 // one window (ncols columns), its W^T
 // partials into the FP32 slab `slab` ([nct * 128][64]).  tm: generic address
-// of the window's tensor map (TMA form); w: the window's segments (register
-// form only).
-template <int NP, bool TMA, bool WY, bool Q8 = false>
+// of the window's tensor map (FEED_TENSOR); wp: the window's segments
+// (FEED_COLUMNS only).
+template <int NP, int FEED, bool WY, bool Q8 = false>
 __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* wp, int ncols,
                                              uint64_t tm, int64_t rb_begin,
                                              int nloc, float* slab, int drain_blocks,
@@ -293,7 +284,6 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
   auto bar = [&](int i) { return S.bars + 8u * (uint32_t)i; };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nct = (ncols + TCOLS - 1) / TCOLS;
-  const int ntile = nloc * nct;
   // Widths and the Psi ring: with Y, W^T tiles of 64 columns and two Psi
   // buffers; without Y, W^T tiles of 64 or 96 columns (l <= 96 in one pass:
   // the Y accumulators' TMEM is free) and four Psi buffers in the shared
@@ -311,9 +301,20 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     return ((i + 1 + (ct * drain_blocks) / kTcMaxTiles) % drain_blocks) == 0 || i == nloc - 1;
   };
 
+  // The producer leaves when its copies have landed, also after a timeout
+  // elsewhere (bounded): nothing writes into shared memory behind the CTA.
+  auto boxes_landed = [&](int u) {
+    const long long t0 = clock64();
+    for (int v = max(u - NST, 0); v < u; ++v)
+      while (!mbar_try(bar(B_RF0 + v % NST), (v / NST) & 1))
+        if (clock64() - t0 > kWaitCycles) {
+          st_volatile_shared(S.abort_flag, 1);
+          return;
+        }
+  };
+
   if (warp < NCONV) {
-    if constexpr (TMA) {
-    // ------------------------------------------------------ converters (TMA)
+    // ------------------------------------------------------------ converters
     // Raw FP32 boxes (32 columns x 128 rows, 512 B per column) arrive in an
     // NST-stage ring; thread (warp w, lane l) splits one column, rows
     // 4(l%8) + 32g of each box into the (single) piece buffer.  The eight
@@ -396,76 +397,6 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     }
     rc.u = U;
     rc.box = X;
-    } else {
-    // ------------------------------------------------------------ converters
-    // A tile is two half tiles of 64 columns; each thread owns 8 columns x 4
-    // rows of a half tile.  The loads of the next half tile are issued before
-    // the current one is split and stored (ping-pong register buffers), with
-    // plain address arithmetic on the window's single segment when it has one.
-    const Window& w = *wp;
-    const int row_off = lane * 4;
-    const bool one_seg = (w.nseg == 1);
-    const float* seg_base = reinterpret_cast<const float*>(w.seg[0].ptr);
-    const int64_t seg_ld = w.seg[0].ld;
-    auto load_half = [&](int64_t r0, int c0, float4 (&v)[8]) {
-      const bool rows_ok = r0 + 3 < a.m;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int c = c0 + j;
-        const float* p = seg_base;
-        if (rows_ok && c < w.ncols)
-          p = one_seg ? seg_base + (int64_t)c * seg_ld + r0 : column_ptr(w, c) + r0;
-        v[j] = __ldcs(reinterpret_cast<const float4*>(p));
-      }
-    };
-    auto store_half = [&](uint32_t pbuf, int64_t r0, int c0, int col_off,
-                          const float4 (&v)[8]) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        float4 x = split_source(a, w, r0, c0 + j, v[j]);
-        if (Q8) x = e4m3_scaled(x, c0 + j < w.ncols ? a.colscale[c0 + j] : 1.f);
-        const uint32_t off = swz((uint32_t)(col_off + j), (uint32_t)row_off, 2048u);
-        const uint32_t h01 = pack_bf16x2(x.x, x.y), h23 = pack_bf16x2(x.z, x.w);
-        st_shared_v2(pbuf + off, h01, h23);
-        if (NP > 1) {
-          const float2 f01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h01));
-          const float2 f23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h23));
-          st_shared_v2(pbuf + PIECE_BYTES + off, pack_bf16x2(x.x - f01.x, x.y - f01.y),
-                       pack_bf16x2(x.z - f23.x, x.w - f23.y));
-        }
-      }
-    };
-    const int c_lo = warp * 8;         // half 0 columns of this warp
-    const int c_hi = 64 + warp * 8;    // half 1 columns
-    float4 bufA[8], bufB[8];
-    if (ntile > 0) load_half(rb_begin * TR + row_off, c_lo, bufA);
-    int tl = 0;   // tile index inside the range; rc.t + tl: the running count
-    bool ok = true;
-    for (int i = 0; i < nloc && ok; ++i) {
-      const int64_t r0 = (rb_begin + i) * TR + row_off;
-      for (int ct = 0; ct < nct; ++ct, ++tl) {
-        const int cbase = ct * TCOLS;
-        load_half(r0, cbase + c_hi, bufB);                       // half 1 of this tile
-        const int t = rc.t + tl, b = t & 1;
-        if (t >= 2 && !mbar_wait(bar(B_FREE0 + b), ((t >> 1) - 1) & 1, S.abort_flag)) {
-          ok = false;
-          break;
-        }
-        const uint32_t pbuf = S.pieces + (uint32_t)b * NP * PIECE_BYTES;
-        store_half(pbuf, r0, cbase + c_lo, c_lo, bufA);          // half 0
-        if (tl + 1 < ntile) {                                     // half 0 of the next tile
-          const bool last_ct = (ct + 1 == nct);
-          load_half(last_ct ? r0 + TR : r0, last_ct ? c_lo : cbase + TCOLS + c_lo, bufA);
-        }
-        store_half(pbuf, r0, cbase + c_hi, c_hi, bufB);          // half 1
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(B_FULL0 + b));
-        if (warp == 0 && lane == 0) TC_TRACE(0, t);
-      }
-    }
-    rc.t += ntile;
-    }
   } else if (warp < MMA_WARP) {
     // -------------------------------------------------------------- epilogue
     const int q = warp - NCONV;           // TMEM lane quarter
@@ -601,7 +532,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     uint32_t wpend = rc.wpend;  // bit ct: tile ct handed to the epilogue, not yet read out
     uint32_t wpar = rc.wpar;    // bit ct: parity of the flushes of tile ct handed out
     const uint32_t idesc_w = lw == 96 ? IDESC_W96 : IDESC_W;
-    int t = rc.t, U = rc.u;
+    int U = rc.u;
     bool ok = true;
     for (int i = 0; i < nloc && ok; ++i) {
       const int g = rc.g + i, pb = g & (npsi - 1), yb = g & 1;
@@ -610,12 +541,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
       tc_fence_after();
       const uint32_t psi_s = psi0 + (uint32_t)pb * psi_bytes;
       const uint32_t ytm = tmem + (uint32_t)(TMEM_Y + yb * LP);
-      for (int ct = 0; ct < nct; ++ct, ++t, U += NP) {
-        const int b = t & 1;
-        if (!TMA && !mbar_wait(bar(B_FULL0 + b), (t >> 1) & 1, S.abort_flag)) {
-          ok = false;
-          break;
-        }
+      for (int ct = 0; ct < nct; ++ct, U += NP) {
         if ((wpend >> ct) & 1u) {   // the epilogue must have read the last flush
           if (!mbar_wait(bar(B_WE0 + ct), ((wpar >> ct) & 1u) ^ 1u, S.abort_flag)) {
             ok = false;
@@ -624,22 +550,19 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
           wpend &= ~(1u << ct);
         }
         tc_fence_after();
-        const uint32_t pbuf = S.pieces + (uint32_t)b * NP * PIECE_BYTES;
         const uint32_t wtm = tmem + (uint32_t)(ct * lw);
         const uint32_t om = S.omega + (uint32_t)ct * OMEGA_TILE_BYTES;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          uint32_t pa = pbuf + (uint32_t)p * PIECE_BYTES;
-          const int u = U + p;   // TMA form: piece unit u in slot u & 1
-          if (TMA) {   // the MMA thread is on the critical path: poll without sleeping
-            if (!mbar_wait_spin(bar(B_FULL0 + (u & 1)), (u >> 1) & 1, S.abort_flag)) {
-              ok = false;
-              break;
-            }
-            TC_TRACE(1, 2 * u);
-            tc_fence_after();
-            pa = S.pieces + (uint32_t)(u & 1) * PIECE_BYTES;
+          const int u = U + p;   // piece unit u in slot u & 1
+          // the MMA thread is on the critical path: poll without sleeping
+          if (!mbar_wait_spin(bar(B_FULL0 + (u & 1)), (u >> 1) & 1, S.abort_flag)) {
+            ok = false;
+            break;
           }
+          TC_TRACE(1, 2 * u);
+          tc_fence_after();
+          const uint32_t pa = S.pieces + (uint32_t)(u & 1) * PIECE_BYTES;
           // Descriptors: the base ones once per piece; the K steps only move
           // the start-address field (address >> 4, bits 0-13), which the
           // constant offsets below never carry out of (shared addresses <
@@ -661,12 +584,11 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
                        (uint32_t)(ct | p | kk));
             }
           }
-          if (TMA) mma_commit(bar(B_FREE0 + (u & 1)));
+          mma_commit(bar(B_FREE0 + (u & 1)));
           TC_TRACE(1, 2 * u + 1);
         }
         if (!ok) break;
         accw |= 1u << ct;
-        if (!TMA) mma_commit(bar(B_FREE0 + b));
         if (drain_due(i, ct)) {   // hand tile ct's partials to the epilogue
           mma_commit(bar(B_WF0 + ct));
           wpar ^= 1u << ct;
@@ -690,16 +612,15 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     }
     rc.done += 1;
     rc.g += nloc;
-    rc.t = t;
     rc.u = U;
     rc.wpar = wpar;
     rc.wpend = wpend;
-  } else if (TMA && warp == PROD_WARP && lane == 0) {
-    // -------------------------------------------------------- TMA producer
+  } else if (FEED == FEED_TENSOR && warp == PROD_WARP && lane == 0) {
+    // -------------------------------------------------- producer, tensor map
     const uint64_t stream_once = policy_evict_first();
     int u = rc.box;
     bool ok = true;
-    for (int t = 0; t < ntile && ok; ++t) {
+    for (int t = 0; t < nloc * nct && ok; ++t) {
       const int i = t / nct, ct = t - i * nct;
       const int row = (int)((rb_begin + i) * TR);
       for (int j = 0; j < 4; ++j, ++u) {
@@ -714,17 +635,64 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
                     bar(B_RF0 + st), stream_once);
       }
     }
+    boxes_landed(u);
+    rc.box = u;
+  } else if (FEED == FEED_COLUMNS && warp >= PROD_WARP) {
+    // -------------------------------------------------- producer, by columns
+    // A warp copies every NPROD-th box column by column, 16 bytes a lane
+    // (cp.async, zero past the matrix' last row and the window's last column;
+    // nothing outside the columns is read); lane l holds the pointers of
+    // columns 32 b + l.  One warp issues a box in about 1900 cycles, so three
+    // take turns.
+    constexpr int NBOX = 4 * kTcMaxTiles;
+    const float* cp[NBOX];   // the lane's columns, at the range's first row
+#pragma unroll
+    for (int b = 0; b < NBOX; ++b)   // (past the window's last column: the first, unread)
+      cp[b] = column_ptr(*wp, 32 * b + lane < ncols ? 32 * b + lane : 0) + rb_begin * TR;
+    const uint64_t stream_once = policy_evict_first();
+    const uint32_t dst0 = S.raw + (uint32_t)lane * 16u;
+    int u = rc.box;
+    bool ok = true;
+    for (int i = 0; i < nloc && ok; ++i) {
+      const int64_t rleft = a.m - (rb_begin + i) * TR - 4 * lane;   // the lane's rows
+      const int bytes = 4 * (int)(rleft < 0 ? 0 : rleft < 4 ? rleft : 4);
+      const int64_t roff = (int64_t)i * TR + (bytes > 0 ? 4 * lane : 0);
+#pragma unroll
+      for (int b = 0; b < NBOX; ++b) {
+        if (b < 4 * nct && ok && u++ % NPROD == warp - PROD_WARP) {   // uniform over the warp
+          const int v = u - 1, st = v % NST;   // this box
+          if (v >= NST) {
+            int free = 1;
+            if (lane == 0)
+              free = mbar_wait(bar(B_RE0 + st), ((v / NST) - 1) & 1, S.abort_flag, 32);
+            ok = __shfl_sync(0xffffffffu, free, 0) != 0;
+          }
+          if (ok) {
+            const uint32_t dst = dst0 + (uint32_t)st * RAW_BYTES;
+            const int ncol = ncols - 32 * b;
+            const unsigned long long mine = reinterpret_cast<unsigned long long>(cp[b]);
+#pragma unroll 8
+            for (int c = 0; c < 32; ++c) {
+              const float* src =
+                  reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, mine, c)) + roff;
+              cp_async_16(dst + (uint32_t)c * (TR * 4), src, c < ncol ? bytes : 0, stream_once);
+            }
+            cp_async_arrive(bar(B_RF0 + st));
+          }
+        }
+      }
+    }
+    if (lane == 0) boxes_landed(u);
     rc.box = u;
   }
 }
 
 // Omega(window, :) as a K-major bf16 B operand of the Y product, resident
 // for the row range.
-template <bool TMA, bool Q8>
+template <bool Q8>
 __device__ __forceinline__ void fill_omega(const Smem& S, const SketchArgs& a, int ncols,
                                            int64_t col_base) {
-  constexpr int NT_ALL = TMA ? NTHREADS_TMA : NTHREADS;
-  for (int e = threadIdx.x; e < kTcMaxTiles * TCOLS * LP; e += NT_ALL) {
+  for (int e = threadIdx.x; e < kTcMaxTiles * TCOLS * LP; e += blockDim.x) {
     const int s = e % LP, c = e / LP;
     float v = 0.f;
     if (s < a.l && c < ncols) v = a.omega[(col_base + c) * a.l + s];
@@ -750,22 +718,22 @@ __device__ __forceinline__ void tmem_free_all(uint32_t tmem) {
 
 // One window of one matrix: CTA b takes the contiguous row blocks
 // [nrb b / G, nrb (b + 1) / G) of the G CTAs, its W^T partials into slab b.
-template <int NP, bool TMA, bool WY, bool Q8>
-__global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
+template <int NP, int FEED, bool WY, bool Q8>
+__global__ void __launch_bounds__(feed_threads(FEED), 1)
     sketch_tc_kernel(const __grid_constant__ SketchArgs a, const __grid_constant__ Window w,
                      int drain_blocks, int* __restrict__ status,
                      const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ uint8_t smem_raw[];
-  const Smem S = carve<NP, TMA>((smem_u32(smem_raw) + 1023u) & ~1023u);
+  const Smem S = carve((smem_u32(smem_raw) + 1023u) & ~1023u);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int64_t nrb = (a.m + TR - 1) / TR;
   const int64_t rb_begin = nrb * blockIdx.x / gridDim.x;
   const int64_t rb_end = nrb * (blockIdx.x + 1) / gridDim.x;
   if (tid == 0) {
     st_volatile_shared(S.abort_flag, 0);
-    init_bars<TMA>(S);
+    init_bars(S, FEED == FEED_COLUMNS ? 32 : 1);
   }
-  if (WY) fill_omega<TMA, Q8>(S, a, w.ncols, w.col_base);
+  if (WY) fill_omega<Q8>(S, a, w.ncols, w.col_base);
   if (warp == MMA_WARP) tmem_alloc_all(S);
   fence_proxy_async();
   tc_fence_before();
@@ -774,7 +742,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(S.tmem_slot) : "memory");
   RoleCounters rc;
-  sketch_roles<NP, TMA, WY, Q8>(a, &w, w.ncols, reinterpret_cast<uint64_t>(&tmap), rb_begin,
+  sketch_roles<NP, FEED, WY, Q8>(a, &w, w.ncols, reinterpret_cast<uint64_t>(&tmap), rb_begin,
                             (int)(rb_end - rb_begin),
                             a.wpart + (int64_t)blockIdx.x * (kTcMaxTiles * TCOLS) *
                                           w_width(a.l, a.want_Y != 0),
@@ -794,7 +762,7 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
                                            const float* __restrict__ slabs, const QrJob& q,
                                            double tol_factor, uint8_t* scratch) {
   const int l = jb.a.l, n = jb.ncols, lw = w_width(l, false);
-  for (int e = threadIdx.x; e < l * n; e += NTHREADS_TMA) {
+  for (int e = threadIdx.x; e < l * n; e += NTHREADS) {
     const int c = e / l, s = e - c * l;
     float hi = 0.f, lo = 0.f;
     for (int q0 = 0; q0 < jb.nitem; q0 += 8) {
@@ -811,14 +779,14 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
   }
   __syncthreads();
   qr::QrShared& sh = *reinterpret_cast<qr::QrShared*>(scratch);
-  qr::cta_pivoted_qr<NTHREADS_TMA>(q.M, q.rows, q.n, q.n, q.k, tol_factor, nullptr, q.R, q.J,
+  qr::cta_pivoted_qr<NTHREADS>(q.M, q.rows, q.n, q.n, q.k, tol_factor, nullptr, q.R, q.J,
                                    q.colpos, q.kout, sh);
   __syncthreads();
   double* r11 = reinterpret_cast<double*>(scratch + 4096);
   double* rdiag = r11 + kLMaxW * kLMaxW;
   int* Js = reinterpret_cast<int*>(rdiag + kLMaxW);
   const int kk = qr::solve_setup(q.R, q.J, q.kout, q.n, r11, Js, rdiag);
-  for (int j = threadIdx.x >> 5; j < q.n; j += NTHREADS_TMA / 32)
+  for (int j = threadIdx.x >> 5; j < q.n; j += NTHREADS / 32)
     qr::solve_column(j, q.R, q.colpos, q.k, kk, q.n, q.P, r11, rdiag);
   __syncthreads();
 }
@@ -842,7 +810,7 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
 // 64 matrices, 82 GB: 21.4 ms with none, 22.3 ms with all.
 // The TMEM stays allocated throughout.  Every wait stays bounded: a CTA that
 // gives up raises its job's problem flag and stops taking items.
-__global__ void __launch_bounds__(NTHREADS_TMA, 1)
+__global__ void __launch_bounds__(NTHREADS, 1)
     sketch_batch_kernel(const BatchJob* __restrict__ jobs, const CUtensorMap* __restrict__ tmaps,
                         const BatchItem* __restrict__ items, const int32_t* __restrict__ order,
                         int nitems, float* __restrict__ slabs, int* __restrict__ counters,
@@ -850,7 +818,7 @@ __global__ void __launch_bounds__(NTHREADS_TMA, 1)
                         int* __restrict__ stat, int drain_blocks) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
-  const Smem S = carve<1, true>((sbase + 1023u) & ~1023u);
+  const Smem S = carve((sbase + 1023u) & ~1023u);
   const uint32_t s_args = (S.abort_flag + 4u + 15u) & ~15u;       // SketchArgs of the job
   const uint32_t s_item = s_args + (uint32_t)sizeof(SketchArgs);   // item index
   const uint32_t s_last = s_item + 4u;   // the item completed a job that is not deferred
@@ -860,7 +828,7 @@ __global__ void __launch_bounds__(NTHREADS_TMA, 1)
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) {
     st_volatile_shared(S.abort_flag, 0);
-    init_bars<true>(S);   // one barrier set for all ranges: phases follow the counters
+    init_bars(S, 1);   // one barrier set for all ranges: phases follow the counters
   }
   if (warp == MMA_WARP) tmem_alloc_all(S);
   tc_fence_before();
@@ -882,16 +850,16 @@ __global__ void __launch_bounds__(NTHREADS_TMA, 1)
       const BatchJob& jb = jobs[item.job];
       const uint32_t* src = reinterpret_cast<const uint32_t*>(&jb.a);
       uint32_t* dst = reinterpret_cast<uint32_t*>(args);
-      for (int e = tid; e < (int)(sizeof(SketchArgs) / 4); e += NTHREADS_TMA) dst[e] = src[e];
+      for (int e = tid; e < (int)(sizeof(SketchArgs) / 4); e += NTHREADS) dst[e] = src[e];
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
       const uint64_t tm = reinterpret_cast<uint64_t>(tmaps + item.job);
       if (jb.np == 2)
-        sketch_roles<2, true, false>(*args, nullptr, jb.ncols, tm, item.rb0, item.nrb,
+        sketch_roles<2, FEED_TENSOR, false>(*args, nullptr, jb.ncols, tm, item.rb0, item.nrb,
                                      slabs + item.slab, drain_blocks, S, tmem, smem_raw, rc);
       else
-        sketch_roles<1, true, false>(*args, nullptr, jb.ncols, tm, item.rb0, item.nrb,
+        sketch_roles<1, FEED_TENSOR, false>(*args, nullptr, jb.ncols, tm, item.rb0, item.nrb,
                                      slabs + item.slab, drain_blocks, S, tmem, smem_raw, rc);
     }
     if (warp >= NCONV && warp < MMA_WARP) __threadfence();   // the slab writes, GPU-wide
@@ -1009,14 +977,14 @@ __global__ void __cluster_dims__(FS_CTAS, 1, 1) __launch_bounds__(FS_THREADS)
   cl.sync();   // no CTA leaves before its maximum is read
 }
 
-template <int NP, bool TMA>
 size_t tc_smem_bytes() {
-  return 1024 + (TMA ? 2u : 2u * NP) * PIECE_BYTES + kTcMaxTiles * OMEGA_TILE_BYTES +
-         2u * PSI_BYTES + (TMA ? NST * RAW_BYTES : 0u) + NBAR * 8 + 16;
+  return 1024 + 2u * PIECE_BYTES + kTcMaxTiles * OMEGA_TILE_BYTES + 2u * PSI_BYTES +
+         NST * RAW_BYTES + NBAR * 8 + 16;
 }
 
 // Tensor map of the window's single segment: rows x columns FP32, boxes of
-// 128 rows x 32 columns, zero fill outside.  False when it cannot be built.
+// 128 rows x 32 columns, zero fill outside.  False when it cannot be built
+// (several segments, or IDSKETCH_SKETCH_TMA=0 asks for the copies by columns).
 bool make_tmap(const SketchArgs& a, const Window& w, CUtensorMap* tm) {
   if (w.nseg != 1) return false;
   const char* env = getenv("IDSKETCH_SKETCH_TMA");
@@ -1024,16 +992,16 @@ bool make_tmap(const SketchArgs& a, const Window& w, CUtensorMap* tm) {
   return make_tmap_f32_2d(w.seg[0].ptr, a.m, w.seg[0].ncols, w.seg[0].ld, TR, 32, tm);
 }
 
-template <int NP, bool TMA, bool WY, bool Q8>
+template <int NP, int FEED, bool WY, bool Q8>
 cudaError_t launch_variant(const SketchArgs& a, const Window& w, int grid, int drain_blocks,
                            int* status, const CUtensorMap& tm, cudaStream_t st,
                            KernelTimer* timer) {
-  const size_t sm = tc_smem_bytes<NP, TMA>();
-  cudaError_t e = cudaFuncSetAttribute(sketch_tc_kernel<NP, TMA, WY, Q8>,
+  const size_t sm = tc_smem_bytes();
+  cudaError_t e = cudaFuncSetAttribute(sketch_tc_kernel<NP, FEED, WY, Q8>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   if (timer && (e = timer->mark(st)) != cudaSuccess) return e;
-  sketch_tc_kernel<NP, TMA, WY, Q8><<<grid, TMA ? NTHREADS_TMA : NTHREADS, sm, st>>>(
+  sketch_tc_kernel<NP, FEED, WY, Q8><<<grid, feed_threads(FEED), sm, st>>>(
       a, w, drain_blocks, status, tm);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (timer) e = timer->mark(st);
@@ -1054,63 +1022,36 @@ extern "C" int idsk_tc_trace_read(long long* host) {
 }
 #endif
 
-cudaError_t launch_sketch_tc(const SketchArgs& a0, const Window& w, int npieces, int nsm,
+cudaError_t launch_sketch_tc(const SketchArgs& a, const Window& w, int npieces, int nsm,
                              int drain_blocks, int* status, cudaStream_t st, KernelTimer* timer) {
   if (w.ncols <= 0) return cudaSuccess;
-  if (w.ncols > kTcMaxTiles * TCOLS || a0.l > kLMaxW || a0.s0 % 10 != 0)
-    return cudaErrorInvalidValue;
+  if (w.ncols > kTcMaxTiles * TCOLS || a.l > kLMaxW) return cudaErrorInvalidValue;
+  if (a.l > LP && a.want_Y) return cudaErrorInvalidValue;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
-  const bool tma = make_tmap(a0, w, &tm);
-  if (a0.l > LP && a0.want_Y) return cudaErrorInvalidValue;
-  if (a0.l > LP && !tma) {
-    if (a0.s0 != 0) return cudaErrorInvalidValue;
-    // a wide sketch (W only) in the register form: one launch per kPassRows
-    // rows of Psi, the coarse rows gathered by the first (the TMA form takes
-    // all l <= 96 rows in one pass)
-    for (int s0 = 0; s0 < a0.l; s0 += kPassRows) {
-      SketchArgs a = a0;
-      a.s0 = s0;
-      a.l = std::min(kPassRows, a0.l - s0);
-      a.W = a0.W + (int64_t)s0 * a0.ldw;
-      if (s0 > 0) a.cg.on = 0;
-      const cudaError_t e = launch_sketch_tc(a, w, npieces, nsm, drain_blocks, status, st, timer);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  }
-  const SketchArgs& a = a0;
+  const bool tensor = make_tmap(a, w, &tm);
   const int64_t nrb = (a.m + TR - 1) / TR;
   const int grid = (int)std::min<int64_t>(nrb, nsm);
   cudaError_t e;
-  auto go = [&](auto np, auto tmaf, auto wy) {
-    return launch_variant<decltype(np)::value, decltype(tmaf)::value, decltype(wy)::value,
-                          false>(a, w, grid, drain_blocks, status, tm, st, timer);
-  };
-  auto go8 = [&](auto tmaf, auto wy) {   // FP8 form: one piece, quantised
-    return launch_variant<1, decltype(tmaf)::value, decltype(wy)::value, true>(
-        a, w, grid, drain_blocks, status, tm, st, timer);
+  auto go = [&](auto np, auto wy, auto q8) {
+    constexpr int NP = decltype(np)::value;
+    constexpr bool WY = decltype(wy)::value, Q8 = decltype(q8)::value;
+    return tensor ? launch_variant<NP, FEED_TENSOR, WY, Q8>(a, w, grid, drain_blocks, status, tm,
+                                                            st, timer)
+                  : launch_variant<NP, FEED_COLUMNS, WY, Q8>(a, w, grid, drain_blocks, status,
+                                                             tm, st, timer);
   };
   using T = std::true_type;
   using F = std::false_type;
   using N1 = std::integral_constant<int, 1>;
   using N2 = std::integral_constant<int, 2>;
-  if (a.fp8) {
+  if (a.fp8) {   // FP8 form: one piece, quantised
     if (npieces != 1 || !a.colscale) return cudaErrorInvalidValue;
-    if (a.want_Y)
-      e = tma ? go8(T(), T()) : go8(F(), T());
-    else
-      e = tma ? go8(T(), F()) : go8(F(), F());
-  } else if (a.want_Y) {
-    if (npieces == 1)
-      e = tma ? go(N1(), T(), T()) : go(N1(), F(), T());
-    else
-      e = tma ? go(N2(), T(), T()) : go(N2(), F(), T());
+    e = a.want_Y ? go(N1(), T(), T()) : go(N1(), F(), T());
+  } else if (npieces == 1) {
+    e = a.want_Y ? go(N1(), T(), F()) : go(N1(), F(), F());
   } else {
-    if (npieces == 1)
-      e = tma ? go(N1(), T(), F()) : go(N1(), F(), F());
-    else
-      e = tma ? go(N2(), T(), F()) : go(N2(), F(), F());
+    e = a.want_Y ? go(N2(), T(), F()) : go(N2(), F(), F());
   }
   if (e != cudaSuccess) return e;
   const int tot = a.l * w.ncols;
@@ -1169,7 +1110,7 @@ cudaError_t launch_coarse_gather(const Window& w, const int64_t* crow, int64_t m
 }
 
 size_t sketch_batch_smem_bytes() {
-  return tc_smem_bytes<1, true>() + 16 + sizeof(SketchArgs) + 16;
+  return tc_smem_bytes() + 16 + sizeof(SketchArgs) + 16;
 }
 
 cudaError_t launch_sketch_batch(const BatchJob* jobs, const CUtensorMap* tmaps,
@@ -1182,7 +1123,7 @@ cudaError_t launch_sketch_batch(const BatchJob* jobs, const CUtensorMap* tmaps,
   cudaError_t e = cudaFuncSetAttribute(sketch_batch_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  sketch_batch_kernel<<<grid, NTHREADS_TMA, sm, st>>>(jobs, tmaps, items, order, nitems, slabs,
+  sketch_batch_kernel<<<grid, NTHREADS, sm, st>>>(jobs, tmaps, items, order, nitems, slabs,
                                                       counters, qjobs, tol_factor, stat,
                                                       drain_blocks);
   count_launches(1);
