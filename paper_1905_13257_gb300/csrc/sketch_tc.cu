@@ -100,10 +100,11 @@ constexpr uint32_t PIECE_BYTES = TR * TCOLS * 2;     // 32 KB
 constexpr uint32_t PSI_BYTES = LP * TR * 2;          // 16 KB
 constexpr uint32_t OMEGA_TILE_BYTES = LP * TCOLS * 2;  // 16 KB
 constexpr int TMEM_COLS = 512;
-constexpr uint32_t IDESC_W = tc::idesc_bf16(128, LP, 0);   // A^T K-major (K = rows)
-constexpr uint32_t IDESC_W96 = tc::idesc_bf16(128, 96, 0);  // the same, 96 sketch rows
-constexpr uint32_t IDESC_Y = tc::idesc_bf16(128, LP, 1);   // A MN-major (M = rows)
+constexpr uint32_t IDESC_W = tc::idesc_bf16(128, LP, 1);   // A^T MN-major (M = columns)
+constexpr uint32_t IDESC_W96 = tc::idesc_bf16(128, 96, 1);  // the same, 96 sketch rows
+constexpr uint32_t IDESC_Y = tc::idesc_bf16(128, LP, 0);   // A K-major (M = rows), in TMEM
 constexpr int TMEM_Y = kTcMaxTiles * LP;             // Y accumulators after W^T
+constexpr int TMEM_A = TMEM_Y + 2 * LP;              // two piece slots of 64 columns
 
 // Optional timeline of CTA 0 (clock64 stamps per role), compiled only when
 // IDSK_TC_TRACE is defined by a profiling harness.
@@ -130,6 +131,7 @@ struct Smem {
   uint32_t omega;    // [kTcMaxTiles][OMEGA_TILE_BYTES]
   uint32_t psi;      // [2][PSI_BYTES]
   uint32_t bars;     // NBAR x 8 bytes
+  uint32_t colexp;   // FP8 form: the columns' scale exponents, one byte each
   uint32_t tmem_slot;
   uint32_t abort_flag;
 };
@@ -179,11 +181,6 @@ __device__ __forceinline__ float2 e4m3x2(float lo, float hi) {
   return __half22float2(*reinterpret_cast<const __half2*>(&h));
 }
 
-__device__ __forceinline__ float4 e4m3_scaled(float4 x, float sc) {
-  const float2 a = e4m3x2(x.x * sc, x.y * sc), b = e4m3x2(x.z * sc, x.w * sc);
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-
 // Psi(0 .. l-1, r) of row r into column rl of a K-major Psi tile (zero past
 // the last row), in groups of ten draws: only the ceil(l / 10) groups that
 // hold rows below l are drawn.  The tile's rows from there to LWT - 1 keep
@@ -223,7 +220,8 @@ __device__ __forceinline__ Smem carve(uint32_t base) {
   S.psi = S.omega + kTcMaxTiles * OMEGA_TILE_BYTES;
   S.raw = S.psi + 2u * PSI_BYTES;
   S.bars = S.raw + NST * RAW_BYTES;
-  S.tmem_slot = S.bars + NBAR * 8u;
+  S.colexp = S.bars + (NBAR * 8u + 15u) / 16u * 16u;
+  S.tmem_slot = S.colexp + kTcMaxTiles * TCOLS;
   S.abort_flag = S.tmem_slot + 4u;
   return S;
 }
@@ -316,15 +314,38 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
   if (warp < NCONV) {
     // ------------------------------------------------------------ converters
     // Raw FP32 boxes (32 columns x 128 rows, 512 B per column) arrive in an
-    // NST-stage ring; thread (warp w, lane l) splits one column, rows
-    // 4(l%8) + 32g of each box into the (single) piece buffer.  The eight
-    // lanes of a quarter warp share a column; the two quarters of each half
-    // warp take columns 4 apart, so that every 8-byte store phase covers all
-    // 32 banks of the 128-byte-swizzled piece (columns c and c + 4 have
-    // disjoint 16-byte chunk positions for rows 0-31).
-    const int cl = (warp >> 1) * 8 + (warp & 1) * 2 + ((lane >> 3) & 1) * 4 + (lane >> 4);
-    const int rq = (lane & 7) * 4;
-    const uint8_t* rawp = smem_raw + (S.raw - smem_u32(smem_raw));
+    // NST-stage ring.  Thread (warp w, lane l) splits row 32 (w % 4) + l of
+    // 16 columns of each box: the 32 lanes read 128 contiguous bytes of a
+    // column, store 16-byte chunks of 8 columns into the swizzled piece, and
+    // (with Y) the same packed pairs into their TMEM lane.
+    const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+    const float* rawp =
+        reinterpret_cast<const float*>(smem_raw + (S.raw - smem_u32(smem_raw))) + half * 16 * TR +
+        row;
+    const uint32_t prow = (uint32_t)((row >> 3) * 2048 + (row & 7) * 128);
+    const uint32_t pchunk = (uint32_t)((half * 2) ^ (row & 7)) << 4;
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + TMEM_A + half * 8;
+    // one box of a piece: 16 columns of the row, packed in pairs
+    auto put = [&](int slot, int j, const uint32_t(&p)[8]) {
+      const uint32_t d = S.pieces + (uint32_t)slot * PIECE_BYTES + prow + (j >> 1) * 1024u;
+      const uint32_t c0 = pchunk ^ ((j & 1) * 64u);
+      st_shared_v4(d + c0, p[0], p[1], p[2], p[3]);
+      st_shared_v4(d + (c0 ^ 16u), p[4], p[5], p[6], p[7]);
+      if (WY) tmem_st8(trow + (uint32_t)(slot * 64 + j * 16), p);
+    };
+    // the whole warp goes on or gives up (its TMEM stores take all lanes)
+    auto wait = [&](int b, uint32_t parity, uint32_t sleep_ns) {
+      return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, S.abort_flag, sleep_ns)) != 0;
+    };
+    auto piece_done = [&](int slot) {
+      if (WY) {
+        tmem_st_wait();
+        tc_fence_before();
+      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(B_FULL0 + slot));
+    };
     int U = rc.u, X = rc.box;
     bool ok = true;
     for (int i = 0; i < nloc && ok; ++i) {
@@ -333,64 +354,61 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
         // (u >> 1)-th use): with NP = 2 the MMAs of one piece run while the
         // converters write the other.
         const int u0 = U, s0 = u0 & 1;
-        if (u0 >= 2 && !mbar_wait(bar(B_FREE0 + s0), ((u0 >> 1) - 1) & 1, S.abort_flag, 16)) {
+        if (u0 >= 2 && !wait(B_FREE0 + s0, ((u0 >> 1) - 1) & 1, 16)) {
           ok = false;
           break;
         }
+        if (WY) tc_fence_after();
         if (warp == 0 && lane == 0) TC_TRACE(0, 4 * u0);
-        const uint32_t hi_buf = S.pieces + (uint32_t)s0 * PIECE_BYTES;
-        uint32_t lo_keep[NP > 1 ? 32 : 1];   // second piece, packed, until its slot frees
+        uint32_t lo[NP > 1 ? 4 : 1][8];   // second piece, packed, until its slot frees
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int xb = X + j, st = xb % NST;
-          if (ok && !mbar_wait(bar(B_RF0 + st), (xb / NST) & 1, S.abort_flag)) ok = false;
+          if (ok) ok = wait(B_RF0 + st, (xb / NST) & 1, 64);
           if (!ok) continue;
-          const float* raw = reinterpret_cast<const float*>(rawp + st * RAW_BYTES);
-          const int cc = 32 * j + cl;              // column inside the tile
-          float sc = 1.f;                          // FP8 form: the column's scale
-          if (Q8 && ct * TCOLS + cc < ncols) sc = a.colscale[ct * TCOLS + cc];
+          const float* raw = rawp + st * (int)(RAW_BYTES / 4);
+          float x[16];
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int rr = 32 * g + rq;
-            float4 x = *reinterpret_cast<const float4*>(raw + cl * TR + rr);
-            if (Q8) x = e4m3_scaled(x, sc);
-            const uint32_t off = swz((uint32_t)cc, (uint32_t)rr, 2048u);
-            const uint32_t h01 = pack_bf16x2(x.x, x.y), h23 = pack_bf16x2(x.z, x.w);
-            st_shared_v2(hi_buf + off, h01, h23);
-            if (NP > 1) {
-              const float2 f01 =
-                  __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h01));
-              const float2 f23 =
-                  __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h23));
-              lo_keep[(j * 4 + g) * 2] = pack_bf16x2(x.x - f01.x, x.y - f01.y);
-              lo_keep[(j * 4 + g) * 2 + 1] = pack_bf16x2(x.z - f23.x, x.w - f23.y);
+          for (int c = 0; c < 16; ++c) x[c] = raw[c * TR];
+          if (Q8) {   // FP8 form: the columns' scales, by their exponents
+            const uint4 e = *reinterpret_cast<const uint4*>(
+                smem_raw + (S.colexp - smem_u32(smem_raw)) + ct * TCOLS + 32 * j + 16 * half);
+            const uint32_t ew[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+            for (int c = 0; c < 16; c += 2) {
+              const uint32_t w2 = ew[c >> 2] >> ((c & 2) * 8);
+              const float2 q = e4m3x2(x[c] * __uint_as_float((w2 & 255u) << 23),
+                                      x[c + 1] * __uint_as_float(((w2 >> 8) & 255u) << 23));
+              x[c] = q.x;
+              x[c + 1] = q.y;
             }
           }
-          __syncwarp();
+          uint32_t hi[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            hi[c] = pack_bf16x2(x[2 * c], x[2 * c + 1]);
+            if (NP > 1)
+              lo[j][c] = pack_bf16x2(x[2 * c] - __uint_as_float(hi[c] << 16),
+                                     x[2 * c + 1] - __uint_as_float(hi[c] & 0xffff0000u));
+          }
+          put(s0, j, hi);
+          __syncwarp();   // after the loads' values are used: every read is done
           if (lane == 0) mbar_arrive(bar(B_RE0 + st));
         }
         if (!ok) break;
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(B_FULL0 + s0));
+        piece_done(s0);
         if (warp == 0 && lane == 0) TC_TRACE(0, 4 * u0 + 1);
         if (NP > 1) {
           const int u1 = u0 + 1, s1 = u1 & 1;   // the other slot
-          if (u1 >= 2 && !mbar_wait(bar(B_FREE0 + s1), ((u1 >> 1) - 1) & 1, S.abort_flag, 16)) {
+          if (u1 >= 2 && !wait(B_FREE0 + s1, ((u1 >> 1) - 1) & 1, 16)) {
             ok = false;
             break;
           }
+          if (WY) tc_fence_after();
           if (warp == 0 && lane == 0) TC_TRACE(0, 4 * u0 + 2);
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int g = 0; g < 4; ++g)
-              st_shared_v2(S.pieces + (uint32_t)s1 * PIECE_BYTES +
-                               swz((uint32_t)(32 * j + cl), (uint32_t)(32 * g + rq), 2048u),
-                           lo_keep[(j * 4 + g) * 2], lo_keep[(j * 4 + g) * 2 + 1]);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(B_FULL0 + s1));
+          for (int j = 0; j < 4; ++j) put(s1, j, lo[j]);
+          piece_done(s1);
         }
         if (warp == 0 && lane == 0) TC_TRACE(0, 4 * u0 + 3);
       }
@@ -568,20 +586,21 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
           // constant offsets below never carry out of (shared addresses <
           // 256 KB), so the single issuing thread spends two integer adds per
           // MMA instead of rebuilding both descriptors.
-          const uint64_t dA = sdesc(pa, 0u, 2048u), dPsi = sdesc(psi_s, 0u, 2048u);
-          const uint64_t dAy = sdesc(pa, 1024u, 2048u), dOm = sdesc(om, 0u, 2048u);
+          const uint64_t dA = sdesc(pa, 1024u, 2048u), dPsi = sdesc(psi_s, 0u, 2048u);
+          const uint64_t dOm = sdesc(om, 0u, 2048u);
+          const uint32_t ta = tmem + (uint32_t)(TMEM_A + (u & 1) * 64);
           const uint32_t acc0 = (accw >> ct) & 1u;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {   // W^T: K = 16 rows per instruction
             const uint64_t ko = (uint64_t)((kk >> 2) * 64 + (kk & 3) * 2);   // bytes >> 4
-            mma_bf16(wtm, dA + ko, dPsi + ko, idesc_w, acc0 | (uint32_t)(p | kk));
+            mma_bf16(wtm, dA + (uint64_t)(kk * 256), dPsi + ko, idesc_w, acc0 | (uint32_t)(p | kk));
           }
           if (wy) {   // without Y the pieces feed the W^T product only
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {   // Y: K = 16 columns per instruction
               const uint64_t ko = (uint64_t)((kk >> 2) * 64 + (kk & 3) * 2);
-              mma_bf16(ytm, dAy + (uint64_t)(kk * 256), dOm + ko, IDESC_Y,
-                       (uint32_t)(ct | p | kk));
+              mma_bf16_ts(ytm, ta + (uint32_t)(kk * 8), dOm + ko, IDESC_Y,
+                          (uint32_t)(ct | p | kk));
             }
           }
           mma_commit(bar(B_FREE0 + (u & 1)));
@@ -733,6 +752,10 @@ __global__ void __launch_bounds__(feed_threads(FEED), 1)
     st_volatile_shared(S.abort_flag, 0);
     init_bars(S, FEED == FEED_COLUMNS ? 32 : 1);
   }
+  if (Q8)
+    for (int c = tid; c < kTcMaxTiles * TCOLS; c += blockDim.x)
+      smem_raw[S.colexp - smem_u32(smem_raw) + c] =
+          c < w.ncols ? (uint8_t)(__float_as_uint(a.colscale[c]) >> 23) : (uint8_t)127;
   if (WY) fill_omega<Q8>(S, a, w.ncols, w.col_base);
   if (warp == MMA_WARP) tmem_alloc_all(S);
   fence_proxy_async();
@@ -979,7 +1002,7 @@ __global__ void __cluster_dims__(FS_CTAS, 1, 1) __launch_bounds__(FS_THREADS)
 
 size_t tc_smem_bytes() {
   return 1024 + 2u * PIECE_BYTES + kTcMaxTiles * OMEGA_TILE_BYTES + 2u * PSI_BYTES +
-         NST * RAW_BYTES + NBAR * 8 + 16;
+         NST * RAW_BYTES + NBAR * 8 + 16 + kTcMaxTiles * TCOLS + 16;
 }
 
 // Tensor map of the window's single segment: rows x columns FP32, boxes of
