@@ -122,14 +122,14 @@ struct SlabSrc {
     float hi[RPT], lo[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) hi[q] = lo[q] = 0.f;
-    const float* src = slabs + (int64_t)j * lw + g;
+    const float* src = slabs + slab_index(j, 0, lw);
     for (int i0 = 0; i0 < nitem; i0 += AHEAD) {
       float x[AHEAD][RPT];
 #pragma unroll
       for (int u = 0; u < AHEAD; ++u) {
         const float* p = src + items[min(i0 + u, nitem - 1)].slab;
 #pragma unroll
-        for (int q = 0; q < RPT; ++q) x[u][q] = g + G * q < lw ? p[G * q] : 0.f;
+        for (int q = 0; q < RPT; ++q) x[u][q] = g + G * q < lw ? p[slab_index(0, g + G * q, lw)] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < AHEAD; ++u)

@@ -114,6 +114,13 @@ struct SketchArgs {
   int32_t fp8;             // FP8-E4M3 form (tensor-core path, one bfloat16 piece)
 };
 
+// Entry (column c of the window, sketch row s) of a W^T slab of width lw: per
+// 128-column tile, groups of four sketch rows, each [128 columns][4], so that
+// the 16-byte reductions of a warp (lane = column) touch 512 contiguous bytes.
+__host__ __device__ constexpr int64_t slab_index(int c, int s, int lw) {
+  return (int64_t)(c >> 7) * 128 * lw + (s >> 2) * 512 + (c & 127) * 4 + (s & 3);
+}
+
 // Width of the tensor-core sketch's W^T accumulators and partial slabs: 64
 // columns, or 96 when Y is not formed and l > 64 (the whole sketch in one
 // pass over A).

@@ -270,7 +270,7 @@ struct RoleCounters {
 
 // The roles of one CTA over row blocks rb_begin .. rb_begin + nloc - 1 of
 // one window (ncols columns), its W^T
-// partials into the FP32 slab `slab` ([nct * 128][64]).  tm: generic address
+// partials into the FP32 slab `slab` (slab_index).  tm: generic address
 // of the window's tensor map (FEED_TENSOR); wp: the window's segments
 // (FEED_COLUMNS only).
 template <int NP, int FEED, bool WY, bool Q8 = false>
@@ -471,19 +471,21 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
         // the tile's 128 x lw partials into registers (32 columns at a
         // time); the accumulator goes back to the MMAs once the last chunk
         // is in registers, and the partials are added to this range's FP32
-        // slab [c][s] (the first flush of a tile stores, later ones add in
-        // L2, four entries per reduction; each slab entry is written by one
-        // thread only, in program order, so the sum has a fixed order)
+        // slab (slab_index; the first flush of a tile stores, later ones add
+        // in L2, four entries per reduction; each slab entry is written by one
+        // thread only, in program order, so the sum has a fixed order).  As
+        // [c][s] rows, each reduction of a warp touched 32 lines: 32
+        // wavefronts of the L1 data pipe, which bounds this kernel.
         const uint64_t keep = policy_evict_last();
-        float* dst = slab + (int64_t)(ct * TCOLS + rl) * lw;
+        float* dst = slab + slab_index(ct * TCOLS + rl, 0, lw);
         const bool first = !((wseen >> ct) & 1u);
         auto put = [&](const float(&v)[32], int c0) {
 #pragma unroll
           for (int j = 0; j < 32; j += 4) {
             if (first)
-              st_v4_f32_hint(dst + c0 + j, v[j], v[j + 1], v[j + 2], v[j + 3], keep);
+              st_v4_f32_hint(dst + slab_index(0, c0 + j, lw), v[j], v[j + 1], v[j + 2], v[j + 3], keep);
             else
-              red_add_v4_f32(dst + c0 + j, v[j], v[j + 1], v[j + 2], v[j + 3], keep);
+              red_add_v4_f32(dst + slab_index(0, c0 + j, lw), v[j], v[j + 1], v[j + 2], v[j + 3], keep);
           }
         };
         float v[2][32];
@@ -510,28 +512,34 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
       if (!wok) break;
       if (q == 0 && lane == 0) TC_TRACE(2, 4 * i);
       if (wy) {   // Y of row block i: accumulator yb
+        const int64_t r = (rb_begin + i) * TR + rl;
+        float* yr = reinterpret_cast<float*>(a.Y) + r;
+        // a later window adds: the old values of half the columns are loaded
+        // before the wait for the products, the other half's before the stores
+        float old[32];
+        auto load_old = [&](int h) {
+          if (a.y_accumulate && r < a.m)
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              old[j] = (h * 32 + j < a.l) ? __ldcs(yr + (int64_t)(h * 32 + j) * a.m) : 0.f;
+        };
+        load_old(0);
         if (!mbar_wait(bar(B_YF0 + yb), (g >> 1) & 1, S.abort_flag, 256)) break;
         tc_fence_after();
         if (q == 0 && lane == 0) TC_TRACE(2, 4 * i + 1);
-        const int64_t r = (rb_begin + i) * TR + rl;
-        float* Y = reinterpret_cast<float*>(a.Y);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float v[32];
           tmem_ld32(tmem + lane_base + (uint32_t)(TMEM_Y + yb * LP + h * 32), v);
+          if (a.y_accumulate) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += old[j];
+          }
+          if (h == 0) load_old(1);
           if (r < a.m) {
-            float* yr = Y + r + (int64_t)(h * 32) * a.m;
-            if (a.y_accumulate) {   // all loads in flight before the stores
-              float old[32];
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                old[j] = (h * 32 + j < a.l) ? __ldcs(yr + (int64_t)j * a.m) : 0.f;
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] += old[j];
-            }
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (h * 32 + j < a.l) __stcs(yr + (int64_t)j * a.m, v[j]);
+              if (h * 32 + j < a.l) __stcs(yr + (int64_t)(h * 32 + j) * a.m, v[j]);
           }
         }
         tc_fence_before();
@@ -785,15 +793,16 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
                                            const float* __restrict__ slabs, const QrJob& q,
                                            double tol_factor, uint8_t* scratch) {
   const int l = jb.a.l, n = jb.ncols, lw = w_width(l, false);
-  for (int e = threadIdx.x; e < l * n; e += NTHREADS) {
-    const int c = e / l, s = e - c * l;
+  for (int e = threadIdx.x; e < (l + 3) / 4 * 4 * n; e += NTHREADS) {
+    const int s = e / (4 * n) * 4 + (e & 3), c = (e >> 2) % n;   // 16-byte groups of columns
+    if (s >= l) continue;
     float hi = 0.f, lo = 0.f;
     for (int q0 = 0; q0 < jb.nitem; q0 += 8) {
       float x[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         x[u] = q0 + u < jb.nitem
-                   ? __ldcg(slabs + items[jb.item0 + q0 + u].slab + (int64_t)c * lw + s)
+                   ? __ldcg(slabs + items[jb.item0 + q0 + u].slab + slab_index(c, s, lw))
                    : 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) df_add(hi, lo, x[u], 0.f);
@@ -922,9 +931,9 @@ __global__ void wpart_reduce_kernel(const float* __restrict__ wpart, int nslab, 
                                     int ncols, int64_t nrb, double* __restrict__ W, int64_t ldw,
                                     int64_t col_base, const float* __restrict__ colscale) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= l * ncols) return;
-  const int c = e / l, s = e - c * l;
-  const float* src = wpart + (int64_t)c * lw + s;
+  const int s = e / (4 * ncols) * 4 + (e & 3), c = (e >> 2) % ncols;   // as the slabs lie
+  if (s >= l) return;
+  const float* src = wpart + slab_index(c, s, lw);
   const int64_t slab = (int64_t)kTcMaxTiles * TCOLS * lw;
   const bool all_rows = nrb >= nslab;   // then every CTA owns at least one row block
   float hi = 0.f, lo = 0.f;
@@ -1077,7 +1086,7 @@ cudaError_t launch_sketch_tc(const SketchArgs& a, const Window& w, int npieces, 
     e = a.want_Y ? go(N2(), T(), F()) : go(N2(), F(), F());
   }
   if (e != cudaSuccess) return e;
-  const int tot = a.l * w.ncols;
+  const int tot = (a.l + 3) / 4 * 4 * w.ncols;
   wpart_reduce_kernel<<<(tot + 255) / 256, 256, 0, st>>>(
       a.wpart, grid, a.l, w_width(a.l, a.want_Y != 0), w.ncols, nrb, a.W, a.ldw, w.col_base,
       a.fp8 ? a.colscale : nullptr);
