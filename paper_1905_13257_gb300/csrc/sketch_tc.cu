@@ -1106,16 +1106,26 @@ __global__ void coarse_rows_kernel(CoarseGeom g, int64_t m, int64_t* __restrict_
 }
 
 // A_c(:, window) = A(crow, window) (Algorithm 5 step 3), exact FP32, right
-// after the window's sketch while its columns are still the caller's:
-// blockIdx.y = column of the window, threads over the coarse rows.
+// after the window's sketch while its columns are still the caller's: threads
+// over the coarse rows, blockIdx.y = group of CPT columns.  Bound by the 32-byte
+// sectors that hold coarse entries; with one column per thread the 8-byte row
+// numbers took twice the bytes of the entries and one load per thread was in
+// flight: a sketch of 4.7M x 1000 (stride 4) 4410 us, with eight 4335 us; an ID
+// of 589,824 x 1000 (stride 2) 4862 and 4728 us.
+template <int CPT>
 __global__ void coarse_gather_kernel(const __grid_constant__ Window w,
                                      const int64_t* __restrict__ crow, int64_t mc,
                                      float* __restrict__ Ac) {
-  const int c = blockIdx.y;
+  const int c0 = blockIdx.y * CPT;
   const int64_t rc = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (rc >= mc) return;
-  const float* col = column_ptr(w, c);
-  Ac[(w.col_base + c) * mc + rc] = col[crow[rc]];
+  const int64_t r = crow[rc];
+  float x[CPT];
+#pragma unroll
+  for (int q = 0; q < CPT; ++q) x[q] = column_ptr(w, min(c0 + q, w.ncols - 1))[r];
+#pragma unroll
+  for (int q = 0; q < CPT; ++q)
+    if (c0 + q < w.ncols) Ac[(w.col_base + c0 + q) * mc + rc] = x[q];
 }
 }  // namespace
 
@@ -1135,8 +1145,14 @@ cudaError_t launch_fp8_scales(const Window& w, int64_t m, float* scale, cudaStre
 cudaError_t launch_coarse_gather(const Window& w, const int64_t* crow, int64_t mc, float* Ac,
                                  cudaStream_t st) {
   if (w.ncols <= 0 || mc <= 0) return cudaSuccess;
-  coarse_gather_kernel<<<dim3((unsigned)((mc + 255) / 256), (unsigned)w.ncols), 256, 0, st>>>(
-      w, crow, mc, Ac);
+  // several columns per thread once that still fills every SM's threads
+  constexpr int CPT = 8;
+  const unsigned gx = (unsigned)((mc + 255) / 256);
+  if (mc * w.ncols >= (int64_t)CPT * 152 * 2048)
+    coarse_gather_kernel<CPT><<<dim3(gx, (unsigned)((w.ncols + CPT - 1) / CPT)), 256, 0, st>>>(
+        w, crow, mc, Ac);
+  else
+    coarse_gather_kernel<1><<<dim3(gx, (unsigned)w.ncols), 256, 0, st>>>(w, crow, mc, Ac);
   count_launches(1);
   return cudaGetLastError();
 }
