@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
     // Kahan accumulators once per chunk), and a division-free running maximum
     // of |e| / |a| kept as the pair (bn, bd) = (|e|, |a|) of the best entry.
     float bn = 0.f, bd = 1.f;
+    const uint32_t never = (uint32_t)(m >> 63);   // 0, which the compiler cannot know
     bool ok = true;
     for (int i = 0; i < nloc && ok; ++i) {
       const int b = i & 1;
@@ -205,10 +206,12 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
         const int cb = c0 + ch * 128 + c4 * 32;
         const bool full = rok && (cb + 31 < n);
         float v[32];
+        int st = 0;
         if constexpr (TMA) {
           // box u of the ring sequence: row block i, column half ch, chunk c4
           // (zero-filled outside the matrix)
-          const int u = i * 8 + 2 * c4 + ch, st = u % NST;
+          const int u = i * 8 + 2 * c4 + ch;
+          st = u % NST;
           if (!mbar_wait(bar(B_RF0 + st), (u / NST) & 1, abort_flag, 64)) {
             ok = false;
             break;
@@ -218,8 +221,6 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
               st * (RAW_BYTES / 4) + q * 32 + lane;
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] = box[j * TR];
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(B_RE0 + st));
         } else if (full) {
           const float* p = A + r + (int64_t)cb * lda;
 #pragma unroll
@@ -255,6 +256,13 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
           bn = better ? ae : bn;
           bd = better ? aa : bd;
         }
+        // The stage goes back when the loads have returned, not when they are
+        // issued: an arrival overtakes loads in flight, and the next box would
+        // overwrite what they read.  The sum of squares needs every value, and
+        // the vote (always true) needs the sum.
+        if constexpr (TMA)
+          if (__all_sync(0xffffffffu, (__float_as_uint(sa) & never) == 0) && lane == 0)
+            mbar_arrive(bar(B_RE0 + st));
         res.add(se);
         tot.add(sa);
       }
