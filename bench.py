@@ -592,7 +592,8 @@ def run_batched(args):
         "data": "synthetic channel fields (seeded), resident in HBM",
         "config": {"workload": f"{len(probs)} channel fields of uneven size in one graph launch "
                                "(one persistent kernel: work-list sketches, each matrix's W "
-                               "sums, QR and solve by the CTA that completes it): "
+                               "sums, QR and solve by the CTA that completes it, long QRs "
+                               "after it by clusters of 8 SMs): "
                                f"m ~ U[50k, {args.batch_max_rows / 1e6:g}M] (3 x 2ny x ny x 2ny), "
                                "n ~ U[64, 512], "
                                f"k ~ U[10, 80], l = k + 10, seeds 1..{len(probs)}, FP32, "

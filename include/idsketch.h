@@ -287,7 +287,9 @@ typedef struct id_batch id_batch;   /* opaque, library-owned */
  * one problem; problems in order of decreasing QR work) are taken from a
  * device counter, and the CTA that completes a problem's last item sums W
  * from the items' partial slabs and runs the problem's pivoted QR and solve
- * for P while the other CTAs go on with later items.  Every other problem
+ * for P while the other CTAs go on with later items; QRs too long to hide
+ * behind the remaining items run after the work list, a cluster of 8 SMs
+ * each (a rule on the problems' sizes).  Every other problem
  * (FP64 data, unaligned columns) keeps its own chain of kernels on a pool of
  * up to 8 worker streams (largest first, to balance the bytes).  cuda_stream: the stream id_batch_run enqueues on (NULL = legacy
  * default stream).  Errors: ID_ERR_INVALID_ARG (NULL, count outside
