@@ -648,6 +648,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) stream_gemv_kernel(
         }
       }
     };
+    const uint32_t never = (uint32_t)(mc >> 63);   // 0, which the compiler cannot know
     int u = 0;
     for (int64_t it = it0; it < it1; ++it, ++u) {
       const int st = u % SG_ST;
@@ -666,8 +667,13 @@ __global__ void __launch_bounds__(SG_THREADS, 1) stream_gemv_kernel(
       const int ncols = n - g * SG_COLS < SG_COLS ? n - g * SG_COLS : SG_COLS;
       const uint8_t* stage = basep + (size_t)st * SG_STAGE;
       for (int r4 = 4 * tid; ok && r4 < rows; r4 += 4 * SG_CONS * 32) quad(stage, ncols, r4);
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(empty0 + 8u * st);
+      // the stage goes back when its values have been used (an arrival can
+      // overtake loads in flight): the vote, always true, needs every sum
+      uint32_t any = 0;
+#pragma unroll
+      for (int q = 0; q < SG_COLS; ++q) any |= __float_as_uint(hi[q]);
+      if (__all_sync(0xffffffffu, (any & never) == 0) && lane == 0)
+        tc::mbar_arrive(empty0 + 8u * st);
     }
     if (cur >= 0) flush(cur);
   }
