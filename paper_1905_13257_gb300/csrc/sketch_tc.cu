@@ -23,11 +23,16 @@
 // are added (round to nearest) into a per-CTA FP32 slab, about 30 partials
 // per entry, and the slabs are summed in FP32 pairs (about 48 bits).
 //
-// Shared-memory layout.  A piece tile is stored in 128-byte-swizzled 1 KB
-// atoms of 8 columns x 64 rows (rows contiguous).  Read as K-major it is the
-// A operand of the W^T product (M = columns, K = rows); read as MN-major it is
-// the A operand of the Y product (M = rows, K = columns): one copy serves both
-// products.  Psi(:, R)^T and Omega(C, :)^T are K-major B operands.
+// Layout of a piece.  In shared memory 128-byte-swizzled 1 KB atoms of 8 rows x
+// 64 columns (columns contiguous), the MN-major A operand of the W^T product
+// (M = columns, K = rows); with Y also in TMEM (lane = row, pairs of columns),
+// the A operand of the Y product (M = rows, K = columns).  Psi(:, R)^T and
+// Omega(C, :)^T are K-major B operands in shared memory.  The TMEM copy is
+// there because the SM's L1 / shared-memory data pipe bounds the kernel with
+// Y: with both A operands from shared memory a tile took 512 wavefronts of
+// incoming boxes, 2173 of loads and stores and 1536 of operands in 4300 clocks;
+// now 512, 1870 and 1024 (4.7M x 1000 in two windows: 4678 -> 4410 us, the
+// slabs' layout below included).
 //
 // Warp roles (one CTA per SM, persistent over a contiguous range of row
 // blocks):

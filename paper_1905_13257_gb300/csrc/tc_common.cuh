@@ -123,16 +123,8 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, uint64_t tmap, int x, 
 }
 
 // Bulk copy (no tensor map) of `bytes` (a multiple of 16) from 16-byte aligned
-// global memory to shared memory, completing on an mbarrier.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
-                                         uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-      ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
-// bulk_g2s with an L2 cache policy (createpolicy) for the source lines.
+// global memory to shared memory, completing on an mbarrier, with an L2 cache
+// policy (createpolicy) for the source lines.
 __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void* src, uint32_t bytes,
                                               uint32_t bar, uint64_t policy) {
   asm volatile(
