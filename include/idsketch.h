@@ -451,6 +451,9 @@ id_status id_timing_read(id_sketch* h, int32_t which, double* total_ms, int64_t*
  *   mode 2: the grid barrier of a cooperative launch of 2 CTAs, one of which
  *           never reaches it                           -> ID_ERR_TIMEOUT
  *   mode 3: the same barrier reached by both CTAs       -> ID_OK
+ *   mode 4: a warp's wait, half of its lanes on a phase that completes and
+ *           half on one that does not: all lanes give up -> ID_ERR_TIMEOUT
+ *   mode 5: the same with both phases completed         -> ID_OK
  * Nothing faults and the context stays usable.  Synchronous (its own
  * stream).  Errors: ID_ERR_INVALID_ARG (mode), ID_ERR_CUDA. */
 id_status id_check_wait(int32_t device, int32_t mode);

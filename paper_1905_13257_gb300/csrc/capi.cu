@@ -786,7 +786,7 @@ id_status id_timing_read(id_sketch* h, int32_t which, double* total_ms, int64_t*
 }
 
 id_status id_check_wait(int32_t device, int32_t mode) {
-  if (mode < 0 || mode > 3) return ID_ERR_INVALID_ARG;
+  if (mode < 0 || mode > 5) return ID_ERR_INVALID_ARG;
   int prev = 0;
   if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(device) != cudaSuccess) {
     g_last_cuda_error.store((int)cudaGetLastError());

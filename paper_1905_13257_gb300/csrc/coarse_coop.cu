@@ -847,6 +847,29 @@ __global__ void mbar_check_kernel(int complete, int* status) {
   if (!tc::mbar_wait<kCheckWaitCycles>(b, 0, af)) atomicOr(status, 1);
 }
 
+// One warp waits as a whole, its lower half on a barrier that completes, its
+// upper half on one that completes only with `complete`: the status is raised
+// when every lane gave up.
+__global__ void mbar_warp_check_kernel(int complete, int* status) {
+  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ int abort_flag;
+  const uint32_t b = tc::smem_u32(&bars[0]), af = tc::smem_u32(&abort_flag);
+  if (threadIdx.x == 0) {
+    tc::mbar_init(b, 1);
+    tc::mbar_init(b + 8, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    tc::mbar_arrive(b);
+    if (complete) tc::mbar_arrive(b + 8);
+  }
+  const bool ok = tc::mbar_wait_warp<kCheckWaitCycles>(b + (threadIdx.x < 16 ? 0u : 8u), 0, af);
+  const unsigned gave = __ballot_sync(0xffffffffu, !ok);
+  if (threadIdx.x == 0 && gave == 0xffffffffu) atomicOr(status, 1);
+}
+
 // The coarse kernel's grid barrier over a cooperative launch; `skip`: the
 // last CTA returns without reaching it.
 __global__ void __launch_bounds__(CT, 1) grid_check_kernel(CoopArgs a, int skip) {
@@ -897,6 +920,9 @@ cudaError_t run_wait_check(int mode, cudaStream_t st, int* gave_up) {
   if ((e = cudaMemsetAsync(words, 0, sizeof(g_check_words), st)) != cudaSuccess) return e;
   if (mode == 0 || mode == 1) {
     mbar_check_kernel<<<1, 32, 0, st>>>(mode == 1, words + 7);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  } else if (mode >= 4) {
+    mbar_warp_check_kernel<<<1, 32, 0, st>>>(mode == 5, words + 7);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else {
     CoopArgs a;

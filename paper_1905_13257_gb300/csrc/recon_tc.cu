@@ -29,7 +29,11 @@
 // and single-buffers the skeleton pieces to make room; the other form loads
 // A in the epilogue warps directly.
 // Waits are bounded as in the sketch kernel; on timeout the status word is
-// set and the host reports ID_ERR_TIMEOUT.
+// set and the host reports ID_ERR_TIMEOUT.  The warps that take part in
+// full-mask or .aligned instructions (votes, tcgen05.ld) keep their loops after
+// a timeout, on whatever data there is and, from the next row block on, without
+// waits: the lanes of a warp poll for themselves, and one that left alone would
+// keep the others waiting without a bound (a vote per wait instead: 2% slower).
 #include <cuda_bf16.h>
 #include <stdlib.h>
 #include <string.h>
@@ -196,9 +200,9 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
     // of |e| / |a| kept as the pair (bn, bd) = (|e|, |a|) of the best entry.
     float bn = 0.f, bd = 1.f;
     const uint32_t never = (uint32_t)(m >> 63);   // 0, which the compiler cannot know
-    bool ok = true;
-    for (int i = 0; i < nloc && ok; ++i) {
+    for (int i = 0; i < nloc; ++i) {
       const int b = i & 1;
+      const bool gone = ld_volatile_shared(abort_flag) != 0;
       const int64_t r = (rb_begin + i) * TR + q * 32 + lane;
       const bool rok = r < m;
 #pragma unroll 1
@@ -212,10 +216,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
           // (zero-filled outside the matrix)
           const int u = i * 8 + 2 * c4 + ch;
           st = u % NST;
-          if (!mbar_wait(bar(B_RF0 + st), (u / NST) & 1, abort_flag, 64)) {
-            ok = false;
-            break;
-          }
+          if (!gone) mbar_wait(bar(B_RF0 + st), (u / NST) & 1, abort_flag, 64);
           const float* box =
               reinterpret_cast<const float*>(smem_raw + (s_raw - smem_u32(smem_raw))) +
               st * (RAW_BYTES / 4) + q * 32 + lane;
@@ -231,10 +232,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
             v[j] = (rok && cb + j < n) ? __ldcs(A + r + (int64_t)(cb + j) * lda) : 0.f;
         }
         if (c4 == 0) {
-          if (!mbar_wait(bar(B_DF0 + b), (i >> 1) & 1, abort_flag, 128)) {
-            ok = false;
-            break;
-          }
+          if (!gone) mbar_wait(bar(B_DF0 + b), (i >> 1) & 1, abort_flag, 128);
           tc_fence_after();
         }
         float d[32];
@@ -266,7 +264,6 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
         res.add(se);
         tot.add(sa);
       }
-      if (!ok) break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_DE0 + b));
@@ -308,9 +305,9 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
         *reinterpret_cast<uint4*>(sbp + p * S_PIECE + off) =
             make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
     };
-    bool gok = true;
-    for (int i = 0; i < nloc && gok; ++i) {
+    for (int i = 0; i < nloc; ++i) {
       const int b = i % NSB, use = i / NSB;
+      const bool gone = ld_volatile_shared(abort_flag) != 0;
       const int64_t r = (rb_begin + i) * TR + rl;
       const bool rok = r < m;
       uint8_t* sbp = sm_gen + (size_t)b * 3u * S_PIECE;
@@ -320,10 +317,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
         float x[KP];
 #pragma unroll
         for (int t = 0; t < KP; ++t) x[t] = (t < k && rok) ? A[r + (int64_t)Js[t] * lda] : 0.f;
-        if (use >= 1 && !mbar_wait(bar(B_SE0 + b), (use - 1) & 1, abort_flag, 64)) {
-          gok = false;
-          break;
-        }
+        if (use >= 1 && !gone) mbar_wait(bar(B_SE0 + b), (use - 1) & 1, abort_flag, 64);
 #pragma unroll
         for (int t0 = 0; t0 < KP; t0 += 8) store8(sbp, t0, x + t0);
       } else {   // single-pass ID: the skeleton row interpolated from the coarse one
@@ -350,10 +344,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
             }
           }
         }
-        if (use >= 1 && !mbar_wait(bar(B_SE0 + b), (use - 1) & 1, abort_flag, 64)) {
-          gok = false;
-          break;
-        }
+        if (use >= 1 && !gone) mbar_wait(bar(B_SE0 + b), (use - 1) & 1, abort_flag, 64);
 #pragma unroll
         for (int t0 = 0; t0 < KP; t0 += 8) store8(sbp, t0, x + t0);
       }

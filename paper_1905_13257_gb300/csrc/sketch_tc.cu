@@ -338,9 +338,8 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
       st_shared_v4(d + (c0 ^ 16u), p[4], p[5], p[6], p[7]);
       if (WY) tmem_st8(trow + (uint32_t)(slot * 64 + j * 16), p);
     };
-    // the whole warp goes on or gives up (its TMEM stores take all lanes)
     auto wait = [&](int b, uint32_t parity, uint32_t sleep_ns) {
-      return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, S.abort_flag, sleep_ns)) != 0;
+      return mbar_wait_warp(bar(b), parity, S.abort_flag, sleep_ns);
     };
     auto piece_done = [&](int slot) {
       if (WY) {
@@ -431,9 +430,8 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     // have completed; false when the wait gave up
     auto gen_psi = [&](int i) {
       const int g = g0 + i, pb = g & (npsi - 1);
-      if (g >= npsi &&
-          !mbar_wait(bar(B_PSIE0 + pb), ((g / npsi) - 1) & 1, S.abort_flag, 256))
-        return false;
+      const bool free =
+          g < npsi || mbar_wait(bar(B_PSIE0 + pb), ((g / npsi) - 1) & 1, S.abort_flag, 256);
       const int64_t r = (rb_begin + i) * TR + rl;
       const uint32_t dst = psi0 + (uint32_t)pb * psi_bytes;
       if (WY || lw == 64)
@@ -441,6 +439,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
       else
         psi_row<96>(a, r, rl, dst);
       fence_proxy_async();
+      if (!__all_sync(0xffffffffu, free)) return false;   // the warp gives up as one
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_PSIF0 + pb));
       return true;
@@ -468,7 +467,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
       bool wok = true;
       for (int ct = 0; ct < nct; ++ct) {
         if (!drain_due(i, ct)) continue;
-        if (!mbar_wait(bar(B_WF0 + ct), (wpar >> ct) & 1u, S.abort_flag, 256)) {
+        if (!mbar_wait_warp(bar(B_WF0 + ct), (wpar >> ct) & 1u, S.abort_flag, 256)) {
           wok = false;
           break;
         }
@@ -529,7 +528,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
               old[j] = (h * 32 + j < a.l) ? __ldcs(yr + (int64_t)(h * 32 + j) * a.m) : 0.f;
         };
         load_old(0);
-        if (!mbar_wait(bar(B_YF0 + yb), (g >> 1) & 1, S.abort_flag, 256)) break;
+        const bool done = mbar_wait(bar(B_YF0 + yb), (g >> 1) & 1, S.abort_flag, 256);
         tc_fence_after();
         if (q == 0 && lane == 0) TC_TRACE(2, 4 * i + 1);
 #pragma unroll
@@ -541,13 +540,14 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
             for (int j = 0; j < 32; ++j) v[j] += old[j];
           }
           if (h == 0) load_old(1);
-          if (r < a.m) {
+          if (done && r < a.m) {
 #pragma unroll
             for (int j = 0; j < 32; ++j)
               if (h * 32 + j < a.l) __stcs(yr + (int64_t)(h * 32 + j) * a.m, v[j]);
           }
         }
         tc_fence_before();
+        if (!__all_sync(0xffffffffu, done)) break;   // the warp gives up as one
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B_YE0 + yb));
       }

@@ -77,6 +77,16 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
   }
 }
 
+// The same wait by a whole warp, with one answer for all lanes: the lanes poll
+// for themselves, so a phase that completes while another role gives up may
+// answer some of them either way, and a full-mask or .aligned instruction
+// (votes, tcgen05.ld) waits without a bound for lanes that went elsewhere.
+template <long long LIMIT = kWaitCycles>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag,
+                                               uint32_t sleep_ns = 64) {
+  return __all_sync(0xffffffffu, mbar_wait<LIMIT>(bar, parity, abort_flag, sleep_ns)) != 0;
+}
+
 // Bounded wait without sleeping between polls (try_wait itself suspends the
 // thread for a while): for waits on the critical path of a streaming loop.
 __device__ inline bool mbar_wait_spin(uint32_t bar, uint32_t parity, uint32_t abort_flag) {
