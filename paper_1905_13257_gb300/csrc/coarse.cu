@@ -600,6 +600,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) stream_gemv_kernel(
                             pol_keep);
         }
       }
+      tc::ring_landed(full0, SG_ST, u, abort_a);
     }
   } else {
     // ---------------------------------------------------------- consumers

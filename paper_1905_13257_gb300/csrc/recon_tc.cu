@@ -408,6 +408,7 @@ __global__ void __launch_bounds__(TMA ? NTHREADS_TMA : NTHREADS, 1)
                     bar(B_RF0 + st), once);
       }
     }
+    ring_landed(bar(B_RF0), NST, u, abort_flag);
   }
   tc_fence_before();
   __syncthreads();

@@ -304,18 +304,6 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
     return ((i + 1 + (ct * drain_blocks) / kTcMaxTiles) % drain_blocks) == 0 || i == nloc - 1;
   };
 
-  // The producer leaves when its copies have landed, also after a timeout
-  // elsewhere (bounded): nothing writes into shared memory behind the CTA.
-  auto boxes_landed = [&](int u) {
-    const long long t0 = clock64();
-    for (int v = max(u - NST, 0); v < u; ++v)
-      while (!mbar_try(bar(B_RF0 + v % NST), (v / NST) & 1))
-        if (clock64() - t0 > kWaitCycles) {
-          st_volatile_shared(S.abort_flag, 1);
-          return;
-        }
-  };
-
   if (warp < NCONV) {
     // ------------------------------------------------------------ converters
     // Raw FP32 boxes (32 columns x 128 rows, 512 B per column) arrive in an
@@ -667,7 +655,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
                     bar(B_RF0 + st), stream_once);
       }
     }
-    boxes_landed(u);
+    ring_landed(bar(B_RF0), NST, u, S.abort_flag);
     rc.box = u;
   } else if (FEED == FEED_COLUMNS && warp >= PROD_WARP) {
     // -------------------------------------------------- producer, by columns
@@ -714,7 +702,7 @@ __device__ __forceinline__ void sketch_roles(const SketchArgs& a, const Window* 
         }
       }
     }
-    if (lane == 0) boxes_landed(u);
+    if (lane == 0) ring_landed(bar(B_RF0), NST, u, S.abort_flag);
     rc.box = u;
   }
 }

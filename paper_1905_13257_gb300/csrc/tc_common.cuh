@@ -103,6 +103,21 @@ __device__ inline bool mbar_wait_spin(uint32_t bar, uint32_t parity, uint32_t ab
   }
 }
 
+// For a producer that leaves, also after a timeout elsewhere: its last copies
+// into a ring of `stages` (full barriers from bar0 on, `copies` issued so far)
+// have landed, so that nothing writes into shared memory behind the CTA.
+// Bounded, with the abort flag raised when it gives up.
+static __device__ __noinline__ void ring_landed(uint32_t bar0, int stages, int copies,
+                                                uint32_t abort_flag) {
+  const long long t0 = clock64();
+  for (int v = copies > stages ? copies - stages : 0; v < copies; ++v)
+    while (!mbar_try(bar0 + 8u * (uint32_t)(v % stages), (uint32_t)(v / stages) & 1u))
+      if (clock64() - t0 > kWaitCycles) {
+        st_volatile_shared(abort_flag, 1);
+        return;
+      }
+}
+
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
