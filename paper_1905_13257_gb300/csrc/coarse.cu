@@ -669,10 +669,11 @@ __global__ void __launch_bounds__(SG_THREADS, 1) stream_gemv_kernel(
       const uint8_t* stage = basep + (size_t)st * SG_STAGE;
       for (int r4 = 4 * tid; ok && r4 < rows; r4 += 4 * SG_CONS * 32) quad(stage, ncols, r4);
       // the stage goes back when its values have been used (an arrival can
-      // overtake loads in flight): the vote, always true, needs every sum
+      // overtake loads in flight): the vote, always true, needs both parts of
+      // every sum (u's low part enters the low parts only)
       uint32_t any = 0;
 #pragma unroll
-      for (int q = 0; q < SG_COLS; ++q) any |= __float_as_uint(hi[q]);
+      for (int q = 0; q < SG_COLS; ++q) any |= __float_as_uint(hi[q]) | __float_as_uint(lo[q]);
       if (__all_sync(0xffffffffu, (any & never) == 0) && lane == 0)
         tc::mbar_arrive(empty0 + 8u * st);
     }
