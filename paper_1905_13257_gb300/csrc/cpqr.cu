@@ -144,7 +144,7 @@ struct SlabSrc {
   }
 };
 
-// Column-pivoted Householder QR of M (rows x n row-major, rows <= 64, n <=
+// Column-pivoted Householder QR of M (rows x n row-major, rows <= LM, n <=
 // 8 * 256 / G) by a cluster of 8 CTAs.  M is only read.
 //
 // What bounds it is not the arithmetic (60 x 1000, k = 50: 5 MFMA) but the
@@ -267,14 +267,36 @@ __device__ __forceinline__ void cluster_qr(const Src& src, int rows, int n, int 
       }
     }
     cl.sync();
-    const Cand& pc = inbox[b][best_of_8(inbox[b], lane)];
+    const int best = best_of_8(inbox[b], lane);
+    const Cand& pc = inbox[b][best];
+    double nrm2 = __longlong_as_double((long long)(pc.key - 1ull));
     if (s == 0) {
       double f = 0.0;
       for (int x = 0; x < CL_CTAS; ++x) f += sh.fro_in[x];
+      const int e2 = (int)((unsigned long long)__double_as_longlong(f) >> 52) - 1023;
+      if (f > 0.0 && e2 < 1024 && (e2 < -800 || e2 > 1000)) {   // uniform over the cluster
+        // data of extreme scale, whose squares (or their reciprocals) leave
+        // FP64's range or lose bits: go on with W times a power of two, which
+        // J and P do not depend on (R is the solve's input only)
+        const double scale = __longlong_as_double((long long)(1023 - e2 / 2) << 52);
+        f = f * scale * scale;
+        if (busy) {
+          ss = 0.0;
+#pragma unroll
+          for (int q = 0; q < RPT; ++q) {
+            c[q] *= scale;
+            ss += c[q] * c[q];
+          }
+          ss = group_sum(ss);
+        }
+        for (int i = t; i < rows; i += CL_THREADS) inbox[b][best].col[i] *= scale;   // own copy
+        __syncthreads();
+        nrm2 = 0.0;
+        for (int i = 0; i < rows; ++i) nrm2 += pc.col[i] * pc.col[i];
+      }
       const double tol = tol_factor * DBL_EPSILON * sqrt(f);
       tol2 = tol * tol;
     }
-    const double nrm2 = __longlong_as_double((long long)(pc.key - 1ull));
     if (pc.key == 0ull || !(nrm2 > tol2)) break;   // uniform over the cluster
     const int p = pc.j;
     double x[RPT], d = 0.0, cs = 0.0;
