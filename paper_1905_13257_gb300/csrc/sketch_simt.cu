@@ -2,7 +2,8 @@
 //
 // One read of each tile of A forms both randomized sketches of the streamed
 // columns (Algorithm 4 step 3, transposed orientation, and eq. eq:sampmatrix):
-//   W(:, cols) = Psi A(:, cols)        (l x ncols, FP64 accumulation)
+//   W(:, cols) = Psi A(:, cols)        (l x ncols; 64-row sums in the data's
+//                                       type, accumulated in FP64)
 //   Y         += A(:, cols) Omega(cols, :)   (m x l)
 // and, when asked, gathers the coarse-grid rows A_c = A(rows_c, cols) of
 // Algorithm 5 step 3 from the same tile.  Psi is never stored: each CTA draws
@@ -15,7 +16,6 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "df.cuh"
 #include "idsk_internal.h"
 
 namespace idsk {
@@ -97,25 +97,18 @@ struct Vec<double> {
   __device__ __forceinline__ double at(int e) const { return e == 0 ? x.x : x.y; }
 };
 
-// W's accumulators: FP64 data adds each tile's sum in FP64; FP32 data as an
-// FP32 pair (about 48 bits: the tile's sum has 24, and GB300's FP64 units, 2
-// operations per clock and SM, would take as long as all the products).
-__device__ __forceinline__ void acc_add(double& w, double v) { w += v; }
-__device__ __forceinline__ void acc_add(float2& w, float v) { df_add(w.x, w.y, v, 0.f); }
-__device__ __forceinline__ double acc_val(double w) { return w; }
-__device__ __forceinline__ double acc_val(float2 w) {   // an infinite sum has no low part
-  return isfinite(w.x) ? df_val(w) : (double)w.x;
+// An FP32 number as FP64 on the integer units: GB300's FP64 units convert at 2
+// a clock and SM, and W's sums keep them busy (315,315 x 333, l = 60: 125 us of
+// the sketch's time).  Zero and normal numbers only.
+__device__ __forceinline__ double widen_normal(float v) {
+  const uint32_t u = __float_as_uint(v), mag = u & 0x7fffffffu;
+  const uint32_t hi = (u & 0x80000000u) | (mag ? (mag >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
 }
-template <typename T>
-struct AccOf;
-template <>
-struct AccOf<float> {
-  using type = float2;
-};
-template <>
-struct AccOf<double> {
-  using type = double;
-};
+__device__ __forceinline__ bool widens(float v) {   // zero or normal
+  const uint32_t x = __float_as_uint(v) << 1;
+  return x == 0u || x - 0x01000000u < 0xfe000000u;
+}
 
 // Shared layout: W accumulators l x ncols | column pointers | coarse rows TM |
 // quantile table | Psi tile 16 SU x kLdt | A tile kTC x kLdt | Omega tile
@@ -144,7 +137,6 @@ __host__ __device__ inline size_t simt_fixed_bytes(int su) {
 template <typename T, int SU>
 __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constant__ SketchArgs a,
                                                             const __grid_constant__ Window w) {
-  using Acc = typename AccOf<T>::type;
   using V = Vec<T>;
   constexpr int TC = kTC<T>, LD = kLdt<T>, LO = 16 * SU;
   constexpr int CU = TC / 16;            // groups of 16 columns in a chunk
@@ -153,7 +145,7 @@ __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constan
   extern __shared__ __align__(16) unsigned char smem[];
   const int ncols = w.ncols, l = a.l;
   const int nacc = (l * ncols + 1) & ~1;   // keeps what follows 16-byte aligned
-  Acc* wacc = reinterpret_cast<Acc*>(smem);
+  double* wacc = reinterpret_cast<double*>(smem);   // W's sums: FP64 over the row tiles
   T* psi_s = reinterpret_cast<T*>(wacc + nacc);
   T* a_s = psi_s + LO * LD;
   T* om_s = a_s + TC * LD;
@@ -165,7 +157,7 @@ __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constan
   const int lr = t & (TM - 1), lc = t / TM;   // loads of A: row, first column
 
   for (int e = t; e < kTableSize; e += NT) tab[e] = a.table[e];
-  for (int e = t; e < l * ncols; e += NT) wacc[e] = Acc{};
+  for (int e = t; e < l * ncols; e += NT) wacc[e] = 0.0;
   for (int c = t; c < ncols; c += NT) {
     const T* p = nullptr;
     for (int q = 0; q < w.nseg; ++q) {
@@ -215,13 +207,28 @@ __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constan
 #pragma unroll
           for (int u = 0; u < CUN; ++u) acc[v][u] += ps[v].at(e) * av[u].at(e);
     }
+    auto add = [&](auto widen) {
 #pragma unroll
-    for (int v = 0; v < SU; ++v)
+      for (int v = 0; v < SU; ++v)
 #pragma unroll
-      for (int u = 0; u < CUN; ++u) {
-        const int sr = ti + 16 * v, c = cc + tj + 16 * u;
-        if (sr < l && c < ncols) acc_add(wacc[sr * ncols + c], acc[v][u]);
-      }
+        for (int u = 0; u < CUN; ++u) {
+          const int sr = ti + 16 * v, c = cc + tj + 16 * u;
+          if (sr < l && c < ncols) wacc[sr * ncols + c] += widen(acc[v][u]);
+        }
+    };
+    if constexpr (sizeof(T) == 4) {
+      bool plain = true;
+#pragma unroll
+      for (int v = 0; v < SU; ++v)
+#pragma unroll
+        for (int u = 0; u < CUN; ++u) plain = plain && widens(acc[v][u]);
+      if (plain)
+        add([](float x) { return widen_normal(x); });
+      else
+        add([](float x) { return (double)x; });
+    } else {
+      add([](double x) { return x; });
+    }
   };
 
   if (blockIdx.x < ntiles) load(blockIdx.x, 0);
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constan
   __syncthreads();
   for (int e = t; e < l * ncols; e += NT) {
     const int sr = e / ncols, c = e % ncols;
-    atomicAdd(&a.W[sr * a.ldw + w.col_base + c], acc_val(wacc[e]));
+    atomicAdd(&a.W[sr * a.ldw + w.col_base + c], wacc[e]);
   }
 }
 
