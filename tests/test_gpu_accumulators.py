@@ -26,3 +26,25 @@ def test_unaligned_sketch_sums_past_fp32_range():
     Wo = P @ A.astype(np.float64)
     assert np.abs(Wo).max() > 4e40
     assert np.max(np.abs(W - Wo)) <= 1e-5 * np.abs(Wo).max()
+
+
+@pytest.mark.parametrize("m,n", [(64, 33), (64, 96), (127, 65)])
+def test_small_fp32_error_pass_keeps_every_square(m, n):
+    """FP32 data with fewer than 128 rows: every square goes into the compensated
+    sums by itself.  A_hat = 1 everywhere, residuals 1 and 2^-12.5 in a pattern of
+    which a chunk's plain FP32 sum loses up to 7 * 2^-25, always downwards.
+    A compensated sum of positive terms is within 2^-25 (the rounding of x - c);
+    numerator and denominator under the root: 2^-25 together."""
+    from paper_1905_13257_gb300 import IdSketch
+    A = np.full((m, n), 1.0 + 2.0 ** -12.5, dtype=np.float32)
+    rows, cols = np.arange(m) % 64 < 16, np.arange(n) % 32 < 16
+    A[np.ix_(rows, cols)] = 2.0
+    A[:, n - 1] = 1.0                       # the skeleton column
+    P = torch.ones((1, n), dtype=torch.float64)
+    sk = IdSketch(m, n, 1, 1, dtype=torch.float32, want_Y=False)
+    fro, _ = sk.reconstruct_error(torch.tensor(A.T.copy(), device="cuda").T,
+                                  torch.tensor([n - 1]), P)
+    sk.close()
+    D = A - np.float32(1.0)                 # exact
+    exact = np.sqrt((D * D).astype(np.float64).sum() / (A * A).astype(np.float64).sum())
+    assert abs(fro - exact) <= 2.0 ** -25 * exact
