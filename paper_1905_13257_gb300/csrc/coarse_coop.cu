@@ -28,11 +28,13 @@
 // 512 rows x 50 columns fill 205 KB; columns that do not fit stay in global
 // memory.
 // Arithmetic: the passes over rows and the sums of their per-CTA partials in
-// FP32 pairs (about 48 bits) for FP32 data, FP64 for the products of FP64 data
-// (V is kept as FP32 pairs for both); scalars, F, R and the norms in FP64;
-// every sum in a fixed order.  GB300's FP64 pipe is narrow (a warp's FP64
-// instruction holds it for about 60 cycles), so nothing per row or per column
-// of a pass over FP32 data runs in FP64.
+// FP32 pairs (about 48 bits) for FP32 data in whole row quads; FP32 data with
+// an odd number of rows: FP32 pairs over a lane's rows, FP64 from there on and
+// for the first norms; FP64 for the products of FP64 data (V is kept as FP32
+// pairs for all); scalars, F, R and the norms in FP64; every sum in a fixed
+// order.  GB300's FP64 pipe is narrow (a warp's FP64 instruction holds it for
+// about 60 cycles), so nothing per row of the steps' passes over FP32 data runs
+// in FP64.
 //
 // Number of CTAs: one per SM for large A_c, at least 16,384 entries each for
 // small ones: a step of a small QR is a chain of latencies, and fewer CTAs
@@ -271,6 +273,12 @@ struct Sum<double> {
   __device__ __forceinline__ double value() const { return v; }
 };
 
+// What lanes' and CTAs' sums are added in, and the column norms formed in: FP32
+// pairs for FP32 data in whole row quads, else FP64 (an odd number of rows: P
+// against 64 bits 3.5e-15 for 42,075 x 333, k = 50, with pairs 5.2e-15).
+template <typename T, bool VEC>
+using Total = Sum<std::conditional_t<VEC, T, double>>;
+
 template <typename S>
 __device__ __forceinline__ void warp_reduce(S& s) {
 #pragma unroll
@@ -298,6 +306,69 @@ __device__ __forceinline__ S reduce4(S (&c)[4], int lane) {
   return keep;
 }
 
+// Sums of four columns' FP32 pairs over the warp, in FP64 (reduce4's lanes), by
+// error-free extraction (S. M. Rump, T. Ogita, S. Oishi, "Accurate
+// floating-point summation", 2008): with 2^B above every lane's |h|, a pair is
+// cut at 2^(B-17) and 2^(B-35) by adding and subtracting 1.5 times a power of
+// two.  32 lanes' first and second slices add up in FP32 without rounding, the
+// third ones within 2^(B-51): as good as FP64 sums of the pairs, whose 10
+// operations hold the FP64 units longer than the pass itself (42,075 x 333, k =
+// 50: a whole ID 3786 us with them, with pairs only 3238 us).
+struct Slices {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(const Slices& o) { a += o.a, b += o.b, c += o.c; }
+  __device__ __forceinline__ Slices from(int mask) const {
+    Slices r;
+    r.a = __shfl_xor_sync(0xffffffffu, a, mask);
+    r.b = __shfl_xor_sync(0xffffffffu, b, mask);
+    r.c = __shfl_xor_sync(0xffffffffu, c, mask);
+    return r;
+  }
+};
+__device__ __forceinline__ Sum<double> reduce4_wide(Sum<float> (&c)[4], int lane) {
+  unsigned e[4];   // exponent of the largest |h|, in every lane
+  bool big = false;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float h = c[q].h + c[q].l, t = h - c[q].h;   // h + l without rounding
+    c[q].l = (c[q].h - (h - t)) + (c[q].l - t);
+    c[q].h = h;
+    e[q] = __reduce_max_sync(0xffffffffu, __float_as_uint(h) & 0x7fffffffu) >> 23;
+    big = big || e[q] > 246u;
+  }
+  Sum<double> r;
+  if (big) {   // (uniform) the first cut would overflow, or has: infinities, NaN
+    Sum<double> d[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q].v = c[q].value();
+    return reduce4(d, lane);
+  }
+  Slices s[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float m1 = __uint_as_float((e[q] + 7u) << 23 | 0x400000u);
+    const float m2 = __uint_as_float((e[q] > 11u ? e[q] - 11u : 1u) << 23 | 0x400000u);
+    s[q].a = __fadd_rn(__fadd_rn(c[q].h, m1), -m1);
+    const float r1 = c[q].h - s[q].a;
+    const float h2 = __fadd_rn(__fadd_rn(r1, m2), -m2), l2 = __fadd_rn(__fadd_rn(c[q].l, m2), -m2);
+    s[q].b = h2 + l2;
+    s[q].c = (r1 - h2) + (c[q].l - l2);
+  }
+  const Slices t = reduce4(s, lane);
+  r.v = (double)t.a + ((double)t.b + (double)t.c);
+  return r;
+}
+// The lanes' sums of four columns, as what they are added in.
+__device__ __forceinline__ void total4(Sum<float> (&c)[4], int lane, Sum<float>& r) {
+  r = reduce4(c, lane);
+}
+__device__ __forceinline__ void total4(Sum<double> (&c)[4], int lane, Sum<double>& r) {
+  r = reduce4(c, lane);
+}
+__device__ __forceinline__ void total4(Sum<float> (&c)[4], int lane, Sum<double>& r) {
+  r = reduce4_wide(c, lane);
+}
+
 // One pass over A_c for the CTA's rows.  Lane l holds rows 4 (l + 32 e) + q
 // (VEC: 128-bit loads, whole row quads) or l + 32 i of every column, RL rows
 // (what the CTA's rows need: the products of lanes without a row cost as much
@@ -307,7 +378,8 @@ __device__ __forceinline__ S reduce4(S (&c)[4], int lane) {
 // evict-last L2 policy.  part: the CTA's n partials.
 template <typename T, bool VEC, int RL>
 struct Pass {
-  using S = Sum<T>;
+  using S = Sum<T>;              // a lane's rows
+  using R = Total<T, VEC>;       // lanes and CTAs
   static constexpr int NB = 2;   // columns in registers
   const T* col0;      // the lane's first row in column 0
   int64_t mc;
@@ -361,21 +433,31 @@ struct Pass {
       for (int i = 0; i < RL; ++i) u[i] = S::u_of(uhs[row0 + off(i)], uls[row0 + off(i)]);
     }
     for (int i0 = 0; i0 < cnt; i0 += 4) {
-      S c[4];
+      std::conditional_t<MODE == 1, S, R> c[4];
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         load(i0 + v + NB - 1, x[(v + NB - 1) % NB]);
-        S sum;
+        if constexpr (MODE == 1) {
 #pragma unroll
-        for (int e = 0; e < RL; ++e) {
-          if (MODE == 1)
-            sum.mac(x[v % NB][e], u[MODE == 1 ? e : 0]);
-          else
-            sum.sq(x[v % NB][e]);
+          for (int e = 0; e < RL; ++e) c[v].mac(x[v % NB][e], u[e]);
+        } else if constexpr (std::is_same_v<S, R>) {
+#pragma unroll
+          for (int e = 0; e < RL; ++e) c[v].sq(x[v % NB][e]);
+        } else {
+          bool plain = true;
+#pragma unroll
+          for (int e = 0; e < RL; ++e) plain = plain && widens(x[v % NB][e]);
+          if (plain) {
+#pragma unroll
+            for (int e = 0; e < RL; ++e) c[v].sq(widen_normal(x[v % NB][e]));
+          } else {
+#pragma unroll
+            for (int e = 0; e < RL; ++e) c[v].sq((double)x[v % NB][e]);
+          }
         }
-        c[v] = sum;
       }
-      const S r = reduce4(c, lane);
+      R r;
+      total4(c, lane, r);
       const int i = i0 + (lane >> 3);
       if ((lane & 7) == 0 && i < cnt) part[warp + CW * i] = r.bits();
     }
@@ -384,7 +466,7 @@ struct Pass {
 
 template <typename T, bool VEC, int RL>
 __global__ void __launch_bounds__(CT, 1) coarse_coop_kernel(CoopArgs a) {
-  using S = Sum<T>;
+  using S = Total<T, VEC>;
   extern __shared__ __align__(16) float2 vs[];   // vs_cols x vs_rows: this CTA's rows of V
   __shared__ int sflag;
   __shared__ __align__(16) float uhs[RMAX];

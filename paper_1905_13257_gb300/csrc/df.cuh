@@ -6,6 +6,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace idsk {
 
@@ -50,6 +51,19 @@ __device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
   e = fmaf(a.x, b.y, e);
   e = fmaf(a.y, b.x, e);
   return df_norm(p, e);
+}
+
+// An FP32 number as FP64 on the integer units: GB300's FP64 units convert at 2
+// a clock and SM (the CUDA-core sketch of 315,315 x 333, l = 60: 125 us of its
+// time).  Zero and normal numbers only.
+__device__ __forceinline__ double widen_normal(float v) {
+  const uint32_t u = __float_as_uint(v), mag = u & 0x7fffffffu;
+  const uint32_t hi = (u & 0x80000000u) | (mag ? (mag >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ bool widens(float v) {   // zero or normal
+  const uint32_t x = __float_as_uint(v) << 1;
+  return x == 0u || x - 0x01000000u < 0xfe000000u;
 }
 
 }  // namespace idsk

@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "df.cuh"
 #include "idsk_internal.h"
 
 namespace idsk {
@@ -96,19 +97,6 @@ struct Vec<double> {
   }
   __device__ __forceinline__ double at(int e) const { return e == 0 ? x.x : x.y; }
 };
-
-// An FP32 number as FP64 on the integer units: GB300's FP64 units convert at 2
-// a clock and SM, and W's sums keep them busy (315,315 x 333, l = 60: 125 us of
-// the sketch's time).  Zero and normal numbers only.
-__device__ __forceinline__ double widen_normal(float v) {
-  const uint32_t u = __float_as_uint(v), mag = u & 0x7fffffffu;
-  const uint32_t hi = (u & 0x80000000u) | (mag ? (mag >> 3) + (896u << 20) : 0u);
-  return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ bool widens(float v) {   // zero or normal
-  const uint32_t x = __float_as_uint(v) << 1;
-  return x == 0u || x - 0x01000000u < 0xfe000000u;
-}
 
 // Shared layout: W accumulators l x ncols | column pointers | coarse rows TM |
 // quantile table | Psi tile 16 SU x kLdt | A tile kTC x kLdt | Omega tile

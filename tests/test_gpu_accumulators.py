@@ -48,3 +48,32 @@ def test_small_fp32_error_pass_keeps_every_square(m, n):
     D = A - np.float32(1.0)                 # exact
     exact = np.sqrt((D * D).astype(np.float64).sum() / (A * A).astype(np.float64).sum())
     assert abs(fro - exact) <= 2.0 ** -25 * exact
+
+
+@pytest.mark.parametrize("mc", [19, 31, 33, 63])
+def test_coarse_products_across_lanes_in_fp64(mc):
+    """FP32 A_c with an odd number of rows, one row per thread: the products are
+    exact FP32 pairs, their sums FP64.  For a column almost orthogonal to the
+    pivot, P's entry is a sum that cancels: within a few roundings (2^-51) of
+    |a_p| |a_j| / |a_p|^2, where sums in FP32 pairs are off by 2^-48."""
+    from paper_1905_13257_gb300 import IdSketch
+    n = 40
+    rng = np.random.default_rng(mc)
+    p = rng.standard_normal(mc)
+    A = rng.standard_normal((mc, n))
+    A -= np.outer(p, p @ A) / (p @ p)
+    A /= np.linalg.norm(A, axis=0)
+    A[:, 7] = 3.0 * p / np.linalg.norm(p)
+    A = A.astype(np.float32)
+    sk = IdSketch(mc, n, 1, 1, dtype=torch.float32, want_Y=False, grid=(1, 1, mc), ncomp=1,
+                  coarse_stride=(1, 1, 1), want_coarse=True)
+    sk.stream_columns(torch.tensor(A.T.copy(), device="cuda").T)
+    J, P, kout = sk.coarse_factor()
+    sk.close()
+    assert kout == 1 and int(J[0]) == 7
+    L = A.astype(np.longdouble)
+    exact = (L[:, 7] @ L) / (L[:, 7] @ L[:, 7])
+    bound = np.linalg.norm(A, axis=0) / np.linalg.norm(A[:, 7]) * 2.0 ** -51
+    off = np.abs(P[0].cpu().numpy() - exact.astype(np.float64)) / bound
+    off[7] = 0.0
+    assert off.max() <= 1.0
