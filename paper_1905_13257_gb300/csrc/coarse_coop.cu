@@ -1083,7 +1083,7 @@ cudaError_t launch_coarse_coop(id_sketch* h, int64_t n64, cudaStream_t st, int m
       n, (int64_t)(std::max(0.0, std::min(1.0, keep)) * l2 / ((double)h->esz * (double)h->mc)));
   a.vrow = reinterpret_cast<float2*>(h->d_hvec);
   a.vs_rows = (int)((Q + G - 1) / G * gran);
-  const size_t room = 227 * 1024 - 8 * 1024;   // static shared memory: about 7 KB
+  constexpr size_t room = kSmemMost - 8 * 1024;   // static shared memory: about 7 KB
   a.vs_cols = (int)std::min<int64_t>(a.kmax, (int64_t)(room / (sizeof(float2) * a.vs_rows)));
   const size_t sm = sizeof(float2) * (size_t)a.vs_cols * a.vs_rows;
   cudaError_t e = cudaMemsetAsync(h->d_cint, 0, 8 * sizeof(int), st);
@@ -1105,7 +1105,7 @@ cudaError_t launch_coarse_coop(id_sketch* h, int64_t n64, cudaStream_t st, int m
            : rl <= 8  ? (const void*)coarse_coop_kernel<float, false, 8>
            : rl <= 12 ? (const void*)coarse_coop_kernel<float, false, 12>
                       : (const void*)coarse_coop_kernel<float, false, 16>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  e = allow_smem(kern, room);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   e = cudaLaunchCooperativeKernel(kern, dim3(G), dim3(CT), args, sm, st);

@@ -409,6 +409,7 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
 // reciprocal, formed once per block), then b_u -= R11(u, t) x_t
 // for u < t, lane u holding b_u and b_{u+32}.  R11 lives in shared memory.
 constexpr int SP_WARPS = 8;
+constexpr size_t kSolveSmem = sizeof(double) * kLMaxW * kLMaxW;   // R11, at most
 __device__ __forceinline__ void solve_p_body(const double* __restrict__ R,
                                              const int* __restrict__ J,
                                              const int* __restrict__ colpos,
@@ -486,8 +487,7 @@ cudaError_t launch_qr_batch(const QrJob* jobs, int njobs, const BatchJob* bjobs,
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t sm = sizeof(double) * (size_t)kmax * kmax;
-  e = cudaFuncSetAttribute(solve_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sm);
+  e = allow_smem(solve_batch_kernel, kSolveSmem);
   if (e != cudaSuccess) return e;
   solve_batch_kernel<<<dim3((nmax + SP_WARPS - 1) / SP_WARPS, njobs), SP_WARPS * 32, sm, st>>>(
       jobs);
@@ -499,8 +499,7 @@ cudaError_t launch_solve_p(const double* R, const int* J, const int* colpos, con
                            int k, int n, double* P, cudaStream_t st) {
   const size_t sm = sizeof(double) * (size_t)k * k;
   if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(solve_p_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = allow_smem(solve_p_kernel, kSolveSmem);
     if (e != cudaSuccess) return e;
   }
   solve_p_kernel<<<(n + SP_WARPS - 1) / SP_WARPS, SP_WARPS * 32, sm, st>>>(R, J, colpos, kout, k,

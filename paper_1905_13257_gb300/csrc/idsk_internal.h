@@ -411,6 +411,15 @@ cudaError_t launch_single_pass_lift(const InterpGeom& g, int64_t m, int dtype, i
                                     cudaStream_t st);
 void gaussian_table_host(float* vals, uint16_t* bits);
 void count_launches(int64_t n);
+// Allows a kernel the most dynamic shared memory that any of its launches takes.
+// The attribute belongs to the kernel, not to a launch: set to a launch's own
+// size, it can be lowered by another thread between this thread's setting and
+// its launch, which then fails.
+template <typename K>
+inline cudaError_t allow_smem(K kern, size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+constexpr size_t kSmemMost = 227 * 1024;   // per CTA
 // Launch the sketch of every pending column window of the handle (capi.cu).
 id_status launch_pending(id_sketch* h);
 // Enqueue the randomized ID of the streamed columns (pivoted QR of W and the

@@ -279,11 +279,12 @@ __global__ void __launch_bounds__(FT) recon_finalize_kernel(const double* __rest
   }
 }
 
+constexpr size_t kReconSmem = 112 * 1024;   // at most
 // All of P in shared memory when two CTAs per SM hold it beside the skeleton
 // rows: no barrier and no load of P per chunk.
 template <typename T>
 bool recon_resident(int k, int64_t n) {
-  return sizeof(T) * (size_t)k * (TM + (size_t)n) <= 112 * 1024;
+  return sizeof(T) * (size_t)k * (TM + (size_t)n) <= kReconSmem;
 }
 template <typename T>
 size_t recon_smem(int k, int64_t n) {
@@ -317,8 +318,7 @@ cudaError_t launch_recon_error(const void* A, int64_t lda, int64_t m, int64_t n,
       (int)std::max<int64_t>(1, std::min<int64_t>((m + TM - 1) / TM, std::min(nblk, 2 * nsm)));
   if (timer && (e = timer->mark(st)) != cudaSuccess) return e;
   auto go = [&](auto kern, const auto* data, size_t sm) {
-    const cudaError_t r =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t r = allow_smem(kern, kReconSmem);
     if (r == cudaSuccess) kern<<<grid, NT, sm, st>>>(data, lda, m, n, J, P, k, part, geo);
     return r;
   };

@@ -162,8 +162,7 @@ cudaError_t launch_single_pass_lift(const InterpGeom& g, int64_t m, int dtype, i
   const unsigned grid = (unsigned)std::min<int64_t>(lines * nseg, 1 << 14);
   auto go = [&](auto kern, auto* out) {
     const size_t sm = sizeof(*out) * (size_t)k * LF_LD;
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = allow_smem(kern, sizeof(*out) * (size_t)kSkelLd * LF_LD);
     if (e == cudaSuccess) kern<<<grid, LF_THREADS, sm, st>>>(g, lines, nseg, m, k, out);
     return e;
   };

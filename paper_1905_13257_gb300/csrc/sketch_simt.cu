@@ -327,8 +327,7 @@ template <typename T>
 cudaError_t launch_simt(const SketchArgs& a, const Window& w, int grid, cudaStream_t st) {
   const size_t sm = simt_smem_bytes<T>(a.l, w.ncols);
   auto go = [&](auto kern) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = allow_smem(kern, kSmemMost);
     if (e != cudaSuccess) return e;
     kern<<<grid, NT, sm, st>>>(a, w);
     return cudaGetLastError();
@@ -358,7 +357,7 @@ cudaError_t launch_gaussian_fill(uint32_t which, uint32_t k0, uint32_t k1, int64
 int simt_window_cols(int l, int dtype) {
   int n = kSimtWindowMax;
   while (n > 16 && (dtype == ID_F64 ? simt_smem_bytes<double>(l, n)
-                                    : simt_smem_bytes<float>(l, n)) > 227 * 1024)
+                                    : simt_smem_bytes<float>(l, n)) > kSmemMost)
     n -= 16;
   return n;
 }
