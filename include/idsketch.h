@@ -345,7 +345,8 @@ id_status id_batch_tune(id_batch* b, int32_t* J, double* P, int32_t* kout, int32
  * P(:, J) = I exactly.  cand: ncand distinct column indices (host or
  * device), 1 <= ncand <= n.  Outputs as id_factor (host or device;
  * synchronises the stream).  Errors: ID_ERR_INVALID_ARG (NULL, ncand out of
- * range, a candidate outside the streamed columns or repeated), ID_ERR_STATE
+ * range, a candidate outside the streamed columns or repeated),
+ * ID_ERR_UNSUPPORTED (l > 64; the handle stays usable), ID_ERR_STATE
  * (no columns yet), ID_ERR_RANK_DEFICIENT (fewer than k pivots above the
  * rank tolerance among the candidates), ID_ERR_TIMEOUT, ID_ERR_CUDA. */
 id_status id_factor_restricted(id_sketch* h, const int32_t* cand, int32_t ncand, int32_t* J,

@@ -549,6 +549,7 @@ id_status id_factor_restricted(id_sketch* h, const int32_t* cand, int32_t ncand,
   if (!h) return ID_ERR_INVALID_ARG;
   if (h->poisoned) return ID_ERR_CUDA;
   if (!cand || ncand < 1) return ID_ERR_INVALID_ARG;
+  if (h->l > kLMax) return ID_ERR_UNSUPPORTED;   // before any work: the handle stays usable
   id_status s = launch_pending(h);
   if (s != ID_OK) return s;
   const int64_t n = h->n_seen;
@@ -566,7 +567,6 @@ id_status id_factor_restricted(id_sketch* h, const int32_t* cand, int32_t ncand,
         return ID_ERR_INVALID_ARG;   // outside the streamed columns, or repeated
   }
   const int k = h->k, l = h->l;
-  if (l > kLMax) IDSK_CUDA(h, cudaErrorInvalidValue);   // restricted form: l <= 64
   // one QR of W over all n columns in which only the candidates may become
   // pivots: R11 and R12 come out together, and P = R11^{-1} R12
   std::vector<int32_t> pos((size_t)n, -1);
