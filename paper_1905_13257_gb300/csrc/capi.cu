@@ -567,16 +567,29 @@ id_status id_factor_restricted(id_sketch* h, const int32_t* cand, int32_t ncand,
         return ID_ERR_INVALID_ARG;   // outside the streamed columns, or repeated
   }
   const int k = h->k, l = h->l;
-  // one QR of W over all n columns in which only the candidates may become
-  // pivots: R11 and R12 come out together, and P = R11^{-1} R12
-  std::vector<int32_t> pos((size_t)n, -1);
-  for (int32_t q = 0; q < ncand; ++q) pos[hc[q]] = q;
-  IDSK_CUDA(h, cudaMemcpyAsync(h->d_cand, pos.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice,
-                               h->st));
-  IDSK_CUDA(h, launch_cpqr_small(h->d_W, h->n_max, h->d_work, l, (int)n, k, ID_RANK_TOL_FACTOR,
-                                 h->d_cand, h->d_R, h->d_J, h->d_colpos, h->d_kout, h->st));
-  IDSK_CUDA(h, launch_solve_p(h->d_R, h->d_J, h->d_colpos, h->d_kout, k, (int)n, h->d_P, h->st));
-  if ((s = copy_out(h, J, h->d_J, sizeof(int32_t) * k)) != ID_OK) return s;
+  std::vector<int32_t> pos;
+  int* d_J = h->d_J;
+  if (cpqr_cluster_ok(l, n)) {
+    // one QR of W over all n columns in which only the candidates may become
+    // pivots: R11 and R12 come out together, and P = R11^{-1} R12
+    pos.assign((size_t)n, -1);
+    for (int32_t q = 0; q < ncand; ++q) pos[hc[q]] = q;
+    IDSK_CUDA(h, cudaMemcpyAsync(h->d_cand, pos.data(), sizeof(int32_t) * n,
+                                 cudaMemcpyHostToDevice, h->st));
+    IDSK_CUDA(h, launch_cpqr_small(h->d_W, h->n_max, h->d_work, l, (int)n, k, ID_RANK_TOL_FACTOR,
+                                   h->d_cand, h->d_R, h->d_J, h->d_colpos, h->d_kout, h->st));
+  } else {
+    // the QR of the candidates, its reflectors applied to all columns; P's
+    // buffer (k n_max >= k (l + 1) doubles here) holds them until the solve
+    d_J = h->d_Jin;
+    IDSK_CUDA(h, cudaMemcpyAsync(h->d_cand, hc.data(), sizeof(int32_t) * ncand,
+                                 cudaMemcpyHostToDevice, h->st));
+    IDSK_CUDA(h, launch_cpqr_columns(h->d_W, h->n_max, h->d_work, l, (int)n, k,
+                                     ID_RANK_TOL_FACTOR, h->d_cand, ncand, h->d_P, h->d_R, h->d_J,
+                                     d_J, h->d_colpos, h->d_kout, h->st));
+  }
+  IDSK_CUDA(h, launch_solve_p(h->d_R, d_J, h->d_colpos, h->d_kout, k, (int)n, h->d_P, h->st));
+  if ((s = copy_out(h, J, d_J, sizeof(int32_t) * k)) != ID_OK) return s;
   if ((s = copy_out(h, P, h->d_P, sizeof(double) * k * n)) != ID_OK) return s;
   int32_t kk = 0, dst = 0;
   IDSK_CUDA(h, cudaMemcpyAsync(&kk, h->d_kout, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st));

@@ -19,11 +19,12 @@
 // columns t, t + 1024, ...
 // In both, sums run in a fixed order.
 //
-// Candidates.  With cpos (one int per column) only the columns with
-// cpos[j] >= 0 may become pivots, ties going to the lowest cpos, and the rank
-// tolerance is that of the candidate columns; every column is updated, so
-// that R11^{-1} R12 is the least-squares fit of all columns on W(:, J)
-// (the learned proposal's restricted ID).
+// Candidates (the learned proposal's restricted ID).  The cluster form with cpos
+// (one int per column): only the columns with cpos[j] >= 0 may become pivots,
+// ties going to the lowest cpos, and the rank tolerance is that of the candidate
+// columns; every column is updated, so that R11^{-1} R12 is the least-squares
+// fit of all columns on W(:, J).  More columns than the cluster holds:
+// launch_cpqr_columns.
 #include <cooperative_groups.h>
 #include <float.h>
 
@@ -43,10 +44,10 @@ constexpr int QMAX = 32;   // columns per thread -> n <= 32768
 
 __global__ void __launch_bounds__(NT, 1)
 cpqr_small_kernel(double* __restrict__ M, int rows, int n, int ld, int k, double tol_factor,
-                  const int* __restrict__ cpos, double* __restrict__ R, int* __restrict__ J,
-                  int* __restrict__ colpos, int* __restrict__ kout) {
+                  double* __restrict__ R, int* __restrict__ J, int* __restrict__ colpos,
+                  int* __restrict__ kout, qr::Reflectors refl) {
   __shared__ qr::QrShared sh;
-  qr::cta_pivoted_qr<NT>(M, rows, n, ld, k, tol_factor, cpos, R, J, colpos, kout, sh);
+  qr::cta_pivoted_qr<NT>(M, rows, n, ld, k, tol_factor, R, J, colpos, kout, sh, refl);
 }
 
 
@@ -99,12 +100,14 @@ __device__ __forceinline__ int best_of_8(const Cand* c, int lane) {
   return (__ffs(__ballot_sync(0xffffffffu, win)) - 1) & 7;
 }
 
-// The matrix of a QR: W itself (row-major) ...
+// The matrix of a QR: W itself (row-major), or columns of it ...
 struct MatrixSrc {
   const double* M;
   int64_t ld;
+  const int* cols = nullptr;
   template <int G, int RPT>
   __device__ __forceinline__ void fill(double (&c)[RPT], int g, int j, int rows) const {
+    if (cols) j = cols[j];
 #pragma unroll
     for (int q = 0; q < RPT; ++q)
       if (g + G * q < rows) c[q] = M[(int64_t)(g + G * q) * ld + j];
@@ -167,12 +170,14 @@ struct SlabSrc {
 // -> 387 us.
 // LM: most rows (64 or 96).  src.fill(c, g, j, rows) loads a lane's rows g, g +
 // G, ... of column j (rows past the last: zero).
-template <int G, int LM, typename Src>
+// KEEP: the reflectors go to refl.
+template <int G, int LM, bool KEEP = false, typename Src>
 __device__ __forceinline__ void cluster_qr(const Src& src, int rows, int n, int k,
                                            double tol_factor,
                                            const int* __restrict__ cpos, double* __restrict__ R,
                                            int* __restrict__ J, int* __restrict__ colpos,
-                                           int* __restrict__ kout, ClusterQr& sh) {
+                                           int* __restrict__ kout, ClusterQr& sh,
+                                           qr::Reflectors refl = {}) {
   constexpr int RPT = LM / G;   // rows per lane
   cg::cluster_group cl = cg::this_cluster();
   cl.barrier_arrive();   // waited for before the first write into another CTA
@@ -338,6 +343,11 @@ __device__ __forceinline__ void cluster_qr(const Src& src, int rows, int n, int 
       cs = __shfl_sync(0xffffffffu, cs, (lane & ~(G - 1)) + gs);
     }
     __syncthreads();
+    if (KEEP && rank == 0 && !worker) {
+      for (int i = s + lane; i < rows; i += 32)
+        refl.V[(int64_t)s * rows + i] = i == s ? sh.v0 : pc.col[i];
+      if (lane == 0) refl.gamma[s] = sh.gamma;
+    }
     if (busy) {
       const double v0 = sh.v0;
       const double w = sh.gamma * (d + v0 * cs);
@@ -369,6 +379,81 @@ __global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
                         int* __restrict__ J, int* __restrict__ colpos, int* __restrict__ kout) {
   __shared__ ClusterQr sh;
   cluster_qr<G, LM>(MatrixSrc{M, ld}, rows, n, k, tol_factor, cpos, R, J, colpos, kout, sh);
+}
+
+// The QR of the columns cols[0 .. n) of M, its reflectors kept (rows <= 64).
+template <int G>
+__global__ void __cluster_dims__(CL_CTAS, 1, 1) __launch_bounds__(CL_THREADS, 1)
+    cpqr_columns_kernel(const double* __restrict__ M, int rows, int n, int64_t ld,
+                        const int* __restrict__ cols, int k, double tol_factor,
+                        double* __restrict__ R, int* __restrict__ J, int* __restrict__ colpos,
+                        int* __restrict__ kout, qr::Reflectors refl) {
+  __shared__ ClusterQr sh;
+  cluster_qr<G, kLMax, true>(MatrixSrc{M, ld, cols}, rows, n, k, tol_factor, nullptr, R, J, colpos,
+                             kout, sh, refl);
+}
+
+// work = M(:, cols), row-major rows x n (the one-CTA QR works in place).
+__global__ void gather_columns_kernel(const double* __restrict__ M, int rows, int n, int64_t ld,
+                                      const int* __restrict__ cols, double* __restrict__ work) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int c = cols[j];
+  for (int i = blockIdx.y; i < rows; i += gridDim.y)
+    work[(int64_t)i * n + j] = M[(int64_t)i * ld + c];
+}
+
+// R(:, j) = the first k_out rows of H_(k_out - 1) ... H_0 M(:, j) for every
+// column j of M (rows <= 64), colpos, and J = cols[Jc]: 16 lanes a column (row i
+// in lane i mod 16), the reflectors in shared memory.
+constexpr int RA_THREADS = 256, RA_COLS = RA_THREADS / 16;
+__global__ void __launch_bounds__(RA_THREADS) reflect_columns_kernel(
+    const double* __restrict__ M, int rows, int n, int64_t ld, const double* __restrict__ V,
+    const double* __restrict__ gamma, const int* __restrict__ cols, const int* __restrict__ Jc,
+    const int* __restrict__ kout, int k, double* __restrict__ R, int* __restrict__ J,
+    int* __restrict__ colpos) {
+  extern __shared__ double vs[];   // k_out x 64, zero outside rows s .. rows - 1
+  __shared__ double gs[kLMax];
+  __shared__ int Js[kLMax];
+  const int kk = *kout, t = threadIdx.x, g = t & 15;
+  for (int e = t; e < kk * kLMax; e += RA_THREADS) {
+    const int s = e / kLMax, i = e % kLMax;
+    vs[e] = i >= s && i < rows ? V[(int64_t)s * rows + i] : 0.0;
+  }
+  for (int u = t; u < kk; u += RA_THREADS) {
+    gs[u] = gamma[u];
+    Js[u] = cols[Jc[u]];
+  }
+  __syncthreads();
+  if (blockIdx.x == 0)
+    for (int u = t; u < k; u += RA_THREADS) J[u] = u < kk ? Js[u] : -1;
+  const int j = blockIdx.x * RA_COLS + (t >> 4);
+  const bool in = j < n;
+  double c[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    c[q] = in && g + 16 * q < rows ? M[(int64_t)(g + 16 * q) * ld + j] : 0.0;
+  int pos = -1;
+  for (int u = g; u < kk; u += 16)
+    if (Js[u] == j) pos = u;
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) pos = max(pos, __shfl_xor_sync(0xffffffffu, pos, o));
+  if (in && g == 0) colpos[j] = pos;
+  for (int s = 0; s < kk; ++s) {
+    const double* v = vs + s * kLMax + g;
+    double d = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q >= s >> 4) d += v[16 * q] * c[q];
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    const double w = gs[s] * d;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= s >> 4) c[q] -= w * v[16 * q];
+      if (in && 16 * q + g == s) R[(int64_t)s * n + j] = c[q];
+    }
+  }
 }
 
 // The slab sums and pivoted QRs of a batch, one cluster per job (n <= 512): all
@@ -451,6 +536,7 @@ cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int ro
                               double tol_factor, const int* cpos, double* R, int* J, int* colpos,
                               int* kout, cudaStream_t st, bool one_cta) {
   if (n > NT * QMAX || rows > kLMaxW || k > kLMaxW) return cudaErrorInvalidValue;
+  if (cpos && !cpqr_cluster_ok(rows, n)) return cudaErrorInvalidValue;
   if (!one_cta && cpqr_cluster_ok(rows, n)) {
     const int cols = (n + CL_CTAS - 1) / CL_CTAS;   // columns per CTA
     auto go = [&](auto kern) {
@@ -471,9 +557,51 @@ cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int ro
         cudaMemcpy2DAsync(work, sizeof(double) * n, W, sizeof(double) * ldw, sizeof(double) * n,
                           rows, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return e;
-    cpqr_small_kernel<<<1, NT, 0, st>>>(work, rows, n, n, k, tol_factor, cpos, R, J, colpos, kout);
+    cpqr_small_kernel<<<1, NT, 0, st>>>(work, rows, n, n, k, tol_factor, R, J, colpos, kout,
+                                        qr::Reflectors{});
   }
   count_launches(1);
+  return cudaGetLastError();
+}
+
+// Candidates of a W with more columns than a cluster holds: the QR of W(:, cand)
+// alone (the cluster form up to 1024 candidates), its reflectors then applied to
+// all columns, whose work spreads over the SMs; the masked QR of all n columns
+// would run in one CTA, in time proportional to n.  Measured, with the solve and
+// the copies of the call (k = 50, l = 60, 100 candidates): n = 4096 404 us in place of
+// 5152 us masked, n = 16,384 786 and 16,848 us.
+cudaError_t launch_cpqr_columns(const double* W, int64_t ldw, double* work, int rows, int n, int k,
+                                double tol_factor, const int* cand, int ncand, double* refl,
+                                double* R, int* Jc, int* J, int* colpos, int* kout,
+                                cudaStream_t st) {
+  if (ncand > NT * QMAX || rows > kLMax || k > kLMax) return cudaErrorInvalidValue;
+  const qr::Reflectors rf{refl, refl + (size_t)k * rows};
+  if (cpqr_cluster_ok(rows, ncand)) {
+    const int per = (ncand + CL_CTAS - 1) / CL_CTAS;   // columns per CTA
+    auto go = [&](auto kern) {
+      kern<<<CL_CTAS, CL_THREADS, 0, st>>>(W, rows, ncand, ldw, cand, k, tol_factor, R, Jc, colpos,
+                                           kout, rf);
+    };
+    if (per <= CL_WORKERS / 16)
+      go(cpqr_columns_kernel<16>);
+    else if (per <= CL_WORKERS / 8)
+      go(cpqr_columns_kernel<8>);
+    else if (per <= CL_WORKERS / 4)
+      go(cpqr_columns_kernel<4>);
+    else
+      go(cpqr_columns_kernel<2>);
+  } else {
+    gather_columns_kernel<<<dim3((ncand + 255) / 256, 8), 256, 0, st>>>(W, rows, ncand, ldw, cand,
+                                                                        work);
+    cpqr_small_kernel<<<1, NT, 0, st>>>(work, rows, ncand, ncand, k, tol_factor, R, Jc, colpos,
+                                        kout, rf);
+    count_launches(1);
+  }
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  reflect_columns_kernel<<<(n + RA_COLS - 1) / RA_COLS, RA_THREADS, sizeof(double) * kLMax * k,
+                           st>>>(W, rows, n, ldw, refl, rf.gamma, cand, Jc, kout, k, R, J, colpos);
+  count_launches(2);
   return cudaGetLastError();
 }
 

@@ -14,8 +14,7 @@ constexpr int kQrCols = 32;   // columns per thread at most (pivot bit mask)
 
 struct ArgMax {
   double v;
-  int i;   // place in the tie order (lowest wins)
-  int j;   // column
+  int i;
 };
 
 __device__ __forceinline__ ArgMax better(ArgMax a, ArgMax b) {
@@ -29,7 +28,6 @@ __device__ __forceinline__ ArgMax warp_argmax(ArgMax a) {
     ArgMax b;
     b.v = __shfl_xor_sync(0xffffffffu, a.v, o);
     b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-    b.j = __shfl_xor_sync(0xffffffffu, a.j, o);
     a = better(a, b);
   }
   return a;
@@ -40,6 +38,13 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+
+// Where a QR leaves its reflectors H_s = I - gamma_s v_s v_s^T: v_s in rows s ..
+// rows - 1 of V(:, s) (leading dimension: the matrix's rows).
+struct Reflectors {
+  double* V = nullptr;
+  double* gamma = nullptr;
+};
 
 // Shared scratch of cta_pivoted_qr (up to 1024 threads).
 struct QrShared {
@@ -54,16 +59,14 @@ struct QrShared {
 // <= 96) by the NT threads of one CTA, in place: thread t owns columns t,
 // t + NT, ... (n <= 32 NT).  k pivots at most; stops early below the rank
 // tolerance tol_factor * eps * ||M||_F.  Writes R (k x n), J (k, -1 past
-// k_out), colpos (n: pivot position or -1) and *kout.  With cpos, only the
-// columns with cpos[j] >= 0 may become pivots (ties to the lowest cpos) and
-// count in ||M||_F.
+// k_out), colpos (n: pivot position or -1) and *kout; with refl.V also the
+// reflectors.
 template <int NT>
 __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows, int n, int ld,
                                                int k, double tol_factor,
-                                               const int* __restrict__ cpos,
                                                double* __restrict__ R, int* __restrict__ J,
                                                int* __restrict__ colpos, int* __restrict__ kout,
-                                               QrShared& sh) {
+                                               QrShared& sh, Reflectors refl = {}) {
   static_assert(NT % 32 == 0 && NT <= 1024, "whole warps, at most 32");
   ArgMax* red = sh.red;
   double* vs = sh.vs;
@@ -86,7 +89,7 @@ __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows,
       if (j >= n) break;
       for (int i = 0; i < rows; ++i) {
         const double x = M[(int64_t)i * ld + j];
-        if (!cpos || cpos[j] >= 0) ss += x * x;
+        ss += x * x;
       }
       colpos[j] = -1;
     }
@@ -104,26 +107,26 @@ __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows,
   int s = 0;
   for (; s < kmax; ++s) {
     // residual norms of the non-pivoted columns
-    ArgMax best{-1.0, 0x7fffffff, -1};
+    ArgMax best{-1.0, 0x7fffffff};
     for (int q = 0; q < kQrCols; ++q) {
       const int j = t + q * NT;
       if (j >= n) break;
-      if ((pivoted & (1u << q)) || (cpos && cpos[j] < 0)) continue;
+      if (pivoted & (1u << q)) continue;
       double ss = 0.0;
       for (int i = s; i < rows; ++i) {
         const double x = M[(int64_t)i * ld + j];
         ss += x * x;
       }
-      best = better(best, ArgMax{ss, cpos ? cpos[j] : j, j});
+      best = better(best, ArgMax{ss, j});
     }
     best = warp_argmax(best);
     if (lane == 0) red[warp] = best;
     __syncthreads();
     if (warp == 0) {
-      ArgMax b = lane < NT / 32 ? red[lane] : ArgMax{-1.0, 0x7fffffff, -1};
+      ArgMax b = lane < NT / 32 ? red[lane] : ArgMax{-1.0, 0x7fffffff};
       b = warp_argmax(b);
       if (lane == 0) {
-        sh_p = b.j;
+        sh_p = b.i;
         sh_stop = !(b.v > sh_tol * sh_tol);
       }
     }
@@ -154,6 +157,11 @@ __device__ __forceinline__ void cta_pivoted_qr(double* __restrict__ M, int rows,
         sh_beta = beta;
         J[s] = p;
         colpos[p] = s;
+      }
+      if (refl.V) {
+        __syncwarp();
+        for (int i = lane; i < len; i += 32) refl.V[(int64_t)s * rows + s + i] = vs[i];
+        if (lane == 0) refl.gamma[s] = tau;
       }
     }
     __syncthreads();

@@ -293,7 +293,7 @@ struct id_sketch {
   int* d_J = nullptr;         // k
   int* d_colpos = nullptr;    // n_max
   int* d_kout = nullptr;      // 1
-  int* d_cand = nullptr;      // n_max: each column's place among the candidates, -1 for none
+  int* d_cand = nullptr;      // n_max: the candidates, or each column's place among them (-1: none)
   // coarse workspace (allocated with the handle when want_coarse)
   double* d_V = nullptr;      // mc x k: reflectors as FP32 pairs (8 bytes each)
   double* d_F = nullptr;      // n_max x k
@@ -376,11 +376,18 @@ cudaError_t launch_qr_batch(const QrJob* jobs, int njobs, const BatchJob* bjobs,
                             double tol_factor, cudaStream_t st);
 // Pivoted QR of W (rows x n row-major, leading dimension ldw) into R (k x n), J,
 // colpos and kout; work: rows x n scratch; cpos: null, or the candidates'
-// places in the tie order (-1: not a candidate).
+// places in the tie order (-1: not a candidate; cluster form only).
 bool cpqr_cluster_ok(int rows, int64_t n);
 cudaError_t launch_cpqr_small(const double* W, int64_t ldw, double* work, int rows, int n, int k,
                               double tol_factor, const int* cpos, double* R, int* J, int* colpos,
                               int* kout, cudaStream_t st, bool one_cta = false);
+// The same for a W of any n <= 32768 columns with the pivots chosen among the
+// columns cand[0 .. ncand): J the pivots' columns of W, colpos for all n; refl: k
+// (rows + 1) doubles of scratch; Jc: the pivots' places among the candidates.
+cudaError_t launch_cpqr_columns(const double* W, int64_t ldw, double* work, int rows, int n, int k,
+                                double tol_factor, const int* cand, int ncand, double* refl,
+                                double* R, int* Jc, int* J, int* colpos, int* kout,
+                                cudaStream_t st);
 cudaError_t launch_solve_p(const double* R, const int* J, const int* colpos, const int* kout,
                            int k, int n, double* P, cudaStream_t st);
 cudaError_t launch_coarse_cpqr(id_sketch* h, int64_t n, cudaStream_t st);

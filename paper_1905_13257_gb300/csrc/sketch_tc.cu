@@ -804,7 +804,7 @@ __device__ __forceinline__ void finish_job(const BatchJob& jb, const BatchItem* 
   }
   __syncthreads();
   qr::QrShared& sh = *reinterpret_cast<qr::QrShared*>(scratch);
-  qr::cta_pivoted_qr<NTHREADS>(q.M, q.rows, q.n, q.n, q.k, tol_factor, nullptr, q.R, q.J,
+  qr::cta_pivoted_qr<NTHREADS>(q.M, q.rows, q.n, q.n, q.k, tol_factor, q.R, q.J,
                                    q.colpos, q.kout, sh);
   __syncthreads();
   double* r11 = reinterpret_cast<double*>(scratch + 4096);
