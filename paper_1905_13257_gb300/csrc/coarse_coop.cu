@@ -1088,13 +1088,20 @@ cudaError_t launch_coarse_coop(id_sketch* h, int64_t n64, cudaStream_t st, int m
   const size_t sm = sizeof(float2) * (size_t)a.vs_cols * a.vs_rows;
   cudaError_t e = cudaMemsetAsync(h->d_cint, 0, 8 * sizeof(int), st);
   if (e != cudaSuccess) return e;
-  // rows per lane of a pass
+  // rows per lane of a pass.  FP64 data is bound by the FP64 units, where a row
+  // that is not there costs as much as one that is: 25,000 x 1000, k = 20 (6 rows)
+  // 3483 us with the 16-row instantiation next after 4, 1728 us with these
+  // (the multi-launch form 3094 us).
   const int rl = (a.vs_rows + 31) / 32;
   const void* kern;
   if (f64)
-    kern = rl <= 1   ? (const void*)coarse_coop_kernel<double, false, 1>
-           : rl <= 4 ? (const void*)coarse_coop_kernel<double, false, 4>
-                     : (const void*)coarse_coop_kernel<double, false, 16>;
+    kern = rl <= 1    ? (const void*)coarse_coop_kernel<double, false, 1>
+           : rl <= 2  ? (const void*)coarse_coop_kernel<double, false, 2>
+           : rl <= 4  ? (const void*)coarse_coop_kernel<double, false, 4>
+           : rl <= 6  ? (const void*)coarse_coop_kernel<double, false, 6>
+           : rl <= 8  ? (const void*)coarse_coop_kernel<double, false, 8>
+           : rl <= 12 ? (const void*)coarse_coop_kernel<double, false, 12>
+                      : (const void*)coarse_coop_kernel<double, false, 16>;
   else if (vec)
     kern = rl <= 4    ? (const void*)coarse_coop_kernel<float, true, 4>
            : rl <= 8  ? (const void*)coarse_coop_kernel<float, true, 8>
