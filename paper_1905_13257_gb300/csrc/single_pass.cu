@@ -58,7 +58,26 @@ __global__ void skeleton_compact_kernel(const T* __restrict__ Ac, int64_t mc,
   Sc[e] = u < k ? Ac[i + (int64_t)Jc[u] * mc] : T(0);
 }
 
-// S = M A_c(:, J_c), column-major m x k, by lines: a line is the nx fine rows
+// S = M A_c(:, J_c), column-major m x k, a fine row per thread: S(r, u) = sum over
+// the 8 corners of w * Sc(corner, u).  For short lines and few columns, where a
+// segment of lift_kernel does too little to pay for its tables and barriers.
+template <typename T>
+__global__ void lift_rows_kernel(InterpGeom g, int64_t m, int k, T* __restrict__ S) {
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= m) return;
+  int64_t idx[8];
+  T w[8];
+  interp_corners<T>(r, g, idx, w);
+  const T* Sc = reinterpret_cast<const T*>(g.Sc);
+  for (int u = 0; u < k; ++u) {
+    T acc = T(0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc += w[q] * Sc[idx[q] * kSkelLd + u];
+    S[r + (int64_t)u * m] = acc;
+  }
+}
+
+// The same by lines: a line is the nx fine rows
 // of one (component, y, z), cut into segments of at most 128.  Per segment the
 // CTA first interpolates in y and z at the coarse x points that the segment
 // touches (lanes along the skeleton's columns: coalesced), into shared memory,
@@ -139,6 +158,20 @@ __global__ void __launch_bounds__(LF_THREADS) lift_kernel(InterpGeom g, int64_t 
   }
 }
 
+// Which form is faster depends on a line's length, its coarse points and k (the
+// number of lines matters to neither), found over nx = 4 to 256, k = 2 to 64,
+// strides 2 and 4 at 0.3 and 1.5 million rows; the whole call in us, by rows and
+// by lines, 1.5 million rows, stride 2:
+//   FP32 nx = 8, k = 24: 390, 627;  nx = 24, k = 8: 227, 257;  k = 16: 368, 265;
+//        nx = 96, k = 2: 123, 150;  k = 40: 913, 228
+//   FP64 nx = 8, k = 64: 1439, 3223;  nx = 32, k = 24: 626, 560;  k = 16: 464, 524;
+//        nx = 128, k = 8: 296, 361;  k = 24: 626, 453
+bool lift_by_rows(const InterpGeom& g, int dtype, int k) {
+  const int64_t nx = g.nx, cx = g.cx;
+  if (dtype == ID_F64) return k * nx < 1000 || k * nx < 28 * cx;
+  return k < 4 || k * cx * cx < 110 * cx + 400;
+}
+
 }  // namespace
 
 cudaError_t launch_skeleton_compact(const void* Ac, int64_t mc, int dtype, const int* Jc, int k,
@@ -157,6 +190,15 @@ cudaError_t launch_skeleton_compact(const void* Ac, int64_t mc, int dtype, const
 
 cudaError_t launch_single_pass_lift(const InterpGeom& g, int64_t m, int dtype, int k, void* S,
                                     cudaStream_t st) {
+  if (lift_by_rows(g, dtype, k)) {
+    const int blocks = (int)((m + 255) / 256);
+    if (dtype == ID_F64)
+      lift_rows_kernel<double><<<blocks, 256, 0, st>>>(g, m, k, reinterpret_cast<double*>(S));
+    else
+      lift_rows_kernel<float><<<blocks, 256, 0, st>>>(g, m, k, reinterpret_cast<float*>(S));
+    count_launches(1);
+    return cudaGetLastError();
+  }
   const int nseg = (g.nx + LF_SEG - 1) / LF_SEG;
   const int64_t lines = m / g.nx;
   const unsigned grid = (unsigned)std::min<int64_t>(lines * nseg, 1 << 14);
