@@ -211,26 +211,38 @@ id_status build_items(id_batch* b, int item_mb) {
   };
   std::stable_sort(jorder.begin(), jorder.end(),
                    [&](int x, int y) { return qr_work(x) > qr_work(y); });
-  // A job is deferred when its QR in one CTA (about 9 us a step and the FP64
-  // work, 3 n (l - s) operations in step s at 2 per clock) takes longer than
-  // the items after it do (about 4 TB/s) -- provided that the longest such
-  // overhang exceeds the cluster QRs themselves (about 6 us a step and 0.1 ms
-  // for their launches).  12 matrices, 2.5 GB, k up to 80: all deferred 1.56 ms
-  // a run, none 3.87 ms; 64 matrices, 82 GB, k from 10 to 79: none deferred
-  // 21.4 ms, the last few 21.5 ms, all 22.3 ms.
-  double after = 0.0, overhang = 0.0, kdef = 0.0;
+  // A job is deferred when its QR in one CTA takes longer than the items after
+  // it do (about 4 TB/s) -- provided that the tail of one-CTA QRs which this
+  // leaves (the longest overhang, or all QRs over all SMs) exceeds the clusters'
+  // (8 SMs each: the longest, or all in rounds of about nsm / 8, and 0.1 ms for
+  // their launches).  Seconds per step, from runs of 19 to 300 matrices (n = 100
+  // to 512, k = 20 to 80): one CTA 11 us and 4.4 n (l - k / 2) FP64 operations at
+  // 2 per nanosecond, a cluster 3.2 us and 11 ns a column.  Both sides, us a run:
+  // matrices          none deferred  all deferred
+  // 12, 2.5 GB, k <= 80    3870       1510
+  // 38 of 1024 x 100, k = 30   492        356
+  // 75 of 1024 x 100, k = 30   493        556
+  // 150 of 1024 x 100, k = 30  495       1059
+  // 75 of 4096 x 512, k = 60  3236       2514
+  // 150 of 1024 x 512, k = 60 3228       4808
+  // 64, 82 GB, k = 10 to 79  21400      22300 (the last few: 21500)
+  double after = 0.0, overhang = 0.0, one_cta = 0.0, longest = 0.0, clusters = 0.0;
   for (auto it = jorder.rbegin(); it != jorder.rend(); ++it) {
     BatchJob& j = b->jobs[*it];
     const double k = b->prob[j.prob].k, l = j.a.l;
-    const double qr_s = k * (9e-6 + 1.5 * j.ncols * (l - 0.5 * k) / 2.0e9);
+    const double qr_s = k * (11e-6 + 4.4 * j.ncols * (l - 0.5 * k) / 2.0e9);
     j.deferred = qr_s > after / 4.0e12 ? 1 : 0;
     if (j.deferred) {
+      const double cl_s = k * (3.2e-6 + 11e-9 * j.ncols);
       overhang = std::max(overhang, qr_s - after / 4.0e12);
-      kdef = std::max(kdef, k);
+      longest = std::max(longest, cl_s);
+      clusters += cl_s * 8.0 / b->nsm;
     }
+    one_cta += qr_s / b->nsm;
     after += 4.0 * (double)j.a.m * j.ncols;
   }
-  if (overhang < 1e-4 + 6e-6 * kdef)
+  if (std::max(overhang, one_cta - after / 4.0e12) <
+      1e-4 + std::max(longest, clusters + 0.5 * longest))
     for (BatchJob& j : b->jobs) j.deferred = 0;
   std::vector<int32_t> order;
   order.reserve(items.size());
