@@ -152,7 +152,6 @@ void build_jobs(id_batch* b) {
       memset(&j, 0, sizeof(j));
       j.a.m = p.m;
       j.a.l = p.l;
-      j.a.lpad = h->lpad;
       j.a.k0 = h->key0;
       j.a.k1 = h->key1;
       j.a.table = h->d_table;

@@ -196,7 +196,6 @@ id_status launch_pending(id_sketch* h) {
     memset(&a, 0, sizeof(a));
     a.m = h->m;
     a.l = h->l;
-    a.lpad = h->lpad;
     a.k0 = h->key0;
     a.k1 = h->key1;
     a.table = h->d_table;
@@ -349,7 +348,6 @@ id_status id_sketch_create(const id_config* cfg, void* cuda_stream, id_sketch** 
   h->n_max = cfg->n_max;
   h->k = cfg->k;
   h->l = cfg->l;
-  h->lpad = ((cfg->l + 15) / 16) * 16;
   h->esz = cfg->dtype == ID_F64 ? 8 : 4;
   h->key0 = (uint32_t)cfg->seed;
   h->key1 = (uint32_t)(cfg->seed >> 32);

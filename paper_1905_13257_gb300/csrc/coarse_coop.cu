@@ -708,13 +708,12 @@ __global__ void __launch_bounds__(CT, 1) coarse_coop_kernel(CoopArgs a) {
     // a fixed order; the last warp takes ||u||^2, the square root and the
     // division while the others sum V_s^T u.
     // The loads that do not depend on the sums go first: u_s, v_t[s] (thread
-    // t < s), and the inputs of this warp's first column of phase C: the CTAs'
-    // partials of (A^T u)_j, F(j, 0:s), A(s, j) and the norm
+    // t < s), and the CTAs' partials of (A^T u)_j and F(j, 0:s) for this warp's
+    // first two columns of phase C
     const float2 us = a.vrow[kLMax];
     const float2 vts = tid < s ? a.vrow[tid] : make_float2(0.f, 0.f);
     struct ColIn {
-      double g[8], f[2], asj, nu2, nu20;   // G <= 256, s <= 64
-      int cp;
+      double g[8], f[2];   // G <= 256, s <= 64
     };
     auto col_in = [&](int j, ColIn& x) {
       const bool on = j < c1;

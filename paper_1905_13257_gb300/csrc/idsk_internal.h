@@ -97,7 +97,7 @@ struct CoarseGeom {
 
 struct SketchArgs {
   int64_t m;
-  int32_t l, lpad;
+  int32_t l;
   uint32_t k0, k1;
   const float* table;   // 4096 quantiles (FP32, bf16-exact)
   const float* omega;   // n_max x l, row-major
@@ -261,7 +261,7 @@ struct id_sketch {
   cudaStream_t st = nullptr;
   int dev = 0, nsm = 0;
   int64_t m = 0, n_max = 0, mc = 0;
-  int k = 0, l = 0, lpad = 0;
+  int k = 0, l = 0;
   size_t esz = 4;
   uint32_t key0 = 0, key1 = 0;
   idsk::CoarseGeom cg{};
