@@ -47,8 +47,9 @@
 // Measured (before: V in global memory, a reduction tree per column, branches
 // around loads, one CTA per SM always; odd m_c and FP64 on four launches per
 // step): 73,728 x 1000, k = 50 on 144 SMs 3.79 -> 3.07 ms; 42,075 x 333, k =
-// 50 about 5.5 -> 1.26 ms; 1152 x 96, k = 8 196 -> 125 us; FP64 1536 x 200,
-// k = 20 about 1 ms -> 330 us.
+// 50 about 5.5 -> 1.26 ms with pair sums throughout, about 0.12 ms more with the
+// wider sums of odd m_c; 1152 x 96, k = 8 196 -> 125 us; FP64 1536 x 200, k = 20
+// about 1 ms -> 330 us.
 // Two columns in registers per warp (three or four were slower: the longer
 // loop costs more in instruction fetch than the loads ahead gain).
 //

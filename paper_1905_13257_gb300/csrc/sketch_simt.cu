@@ -121,7 +121,8 @@ __host__ __device__ inline size_t simt_fixed_bytes(int su) {
 // FP32 data: by the shared-memory bandwidth of the 4 x 4 blocks (512 bytes a
 // warp for every 16 products of a lane, twice the FP32 units' time).
 // Measured: 98,304 x 200 FP64, l = 30 with Y in 7 launches: 8844 -> 2598 us;
-// 315,315 x 333 FP32, l = 60 with Y: 3967 -> 1394 us.
+// 315,315 x 333 FP32, l = 60 with Y: 3967 -> 1394 us with W's sums as FP32
+// pairs, about 100 us more with the FP64 sums they have.
 template <typename T, int SU>
 __global__ void __launch_bounds__(NT, 1) sketch_simt_kernel(const __grid_constant__ SketchArgs a,
                                                             const __grid_constant__ Window w) {
